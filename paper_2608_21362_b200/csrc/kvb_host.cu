@@ -731,19 +731,28 @@ int kvb_quantize_chunks(kvb_ctx* c, const kvb_quantize_job* jobs, int n_jobs, vo
   }
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   KVB_CUDA(c, cudaSetDevice(c->device));
-  uint8_t* host = nullptr;
-  const int slot_code = take_slot(c, &host);
-  if (slot_code >= 0) return slot_code;
-  const int slot = -slot_code - 1;
-  QuantJob* qj = reinterpret_cast<QuantJob*>(host);
-  for (int i = 0; i < n_jobs; ++i) {
-    const kvb_quantize_job& j = jobs[i];
-    qj[i] = QuantJob{j.k, j.v, j.k_codes, j.v_codes, j.k_meta, j.v_meta, j.bits, j.unrotate_from, j.meta_fp16, 0};
+  auto fill = [&](QuantJob* qj) {
+    for (int i = 0; i < n_jobs; ++i) {
+      const kvb_quantize_job& j = jobs[i];
+      qj[i] = QuantJob{j.k, j.v, j.k_codes, j.v_codes, j.k_meta, j.v_meta, j.bits, j.unrotate_from, j.meta_fp16, 0};
+    }
+  };
+  if (n_jobs <= kQuantInline && !c->force_copy) {  // the jobs travel as the kernel's argument
+    QuantJob qj[kQuantInline];
+    fill(qj);
+    c->last_stream = st;
+    KVB_CUDA(c, launch_quantize_inline(qj, n_jobs, c->dims, c->inv_freq, c->status_dev, c->n_sm, c->pdl, st));
+  } else {
+    uint8_t* host = nullptr;
+    const int slot_code = take_slot(c, &host);
+    if (slot_code >= 0) return slot_code;
+    const int slot = -slot_code - 1;
+    fill(reinterpret_cast<QuantJob*>(host));
+    const int up = upload(c, slot, host, sizeof(QuantJob) * (size_t)n_jobs, st);
+    if (up != KVB_OK) return up;
+    c->last_stream = st;
+    KVB_CUDA(c, launch_quantize_table(reinterpret_cast<const QuantJob*>(c->arena_dev), n_jobs, c->dims, c->inv_freq, c->status_dev, c->n_sm, c->pdl, st));
   }
-  const int up = upload(c, slot, host, sizeof(QuantJob) * (size_t)n_jobs, st);
-  if (up != KVB_OK) return up;
-  c->last_stream = st;
-  KVB_CUDA(c, launch_quantize_batch(reinterpret_cast<const QuantJob*>(c->arena_dev), n_jobs, c->dims, c->inv_freq, c->status_dev, c->pdl, st));
   c->launches += 1;
   return KVB_OK;
 }

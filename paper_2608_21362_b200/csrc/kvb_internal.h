@@ -147,9 +147,13 @@ struct QuantJob {
   int32_t meta16;
   int32_t reserved;
 };
-// inv_freq: [d/2] doubles, device
-cudaError_t launch_quantize_batch(const QuantJob* jobs, int n_jobs, const ModelDims& m, const double* inv_freq,
-                                  uint32_t* status, bool pdl, cudaStream_t st);
+// Up to kQuantInline jobs travel as the kernel's own argument (host_jobs is read before the call returns),
+// more through a table in device memory.  inv_freq: [d/2] doubles, device.
+constexpr int kQuantInline = (int)(kDescBlobBytes / sizeof(QuantJob));
+cudaError_t launch_quantize_inline(const QuantJob* host_jobs, int n_jobs, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl,
+                                   cudaStream_t st);
+cudaError_t launch_quantize_table(const QuantJob* table, int n_jobs, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl,
+                                  cudaStream_t st);
 cudaError_t quantize_configure();
 
 }  // namespace kvb

@@ -174,3 +174,56 @@ def test_batched_quantiser_codes_bit_exact(kv_dtype, Hkv):
         assert B.kvb_quantize_chunks(ctx, []) == B.KVB_OK
     finally:
         B.kvb_destroy(ctx)
+
+
+def _eq6(x, bits):
+    """Eq. 6 on [..., group] rows in float32, as the library states it: (codes, scale, min)."""
+    x = x.float()
+    mn, mx = x.amin(-1, keepdim=True), x.amax(-1, keepdim=True)
+    s = torch.where(mx > mn, (mx - mn) / float(2**bits - 1), torch.ones_like(mn))
+    return torch.clamp(torch.round((x - mn) / s), 0, 2**bits - 1), s, mn
+
+
+@pytest.mark.parametrize("n_jobs,L,Hkv,bits", [(1, 1, 1, 8), (60, 1, 2, 4), (61, 1, 2, 8), (256, 1, 1, 4), (257, 1, 2, 8), (3, 5, 4, 4)])
+def test_job_counts_and_extreme_ranges(n_jobs, L, Hkv, bits):
+    """Both argument sizes and the table beyond them, fewer tiles than SMs and ranges that do not divide, and channels
+    whose range is zero, tiny (below the reciprocal's range), huge or ordinary: codes and metadata bit for bit."""
+    sh = synth.Shape(L=L, Hq=Hkv, Hkv=Hkv)
+    ctx = B.create_for_shape(sh, 0, max_chunks_total=512)
+    try:
+        g = torch.Generator().manual_seed(n_jobs)
+        k = torch.randn((n_jobs, L, sh.C, Hkv, sh.d), generator=g)
+        v = torch.randn((n_jobs, L, sh.C, Hkv, sh.d), generator=g)
+        k[..., 5] = 1.5                    # no range
+        k[..., 6] *= 1e-30                 # scale below 1e-20
+        k[..., 70] *= 1e30                 # scale above 1e20
+        k[..., 71] = torch.round(k[..., 71] * 4)  # a coarse lattice: ties
+        v[:, :, 3] *= 1e-30
+        v[:, :, 4] *= 1e30
+        v[:, :, 5] = -2.0
+        k, v = k.to(sh.torch_dtype), v.to(sh.torch_dtype)
+        G = 1 if bits == 8 else 4
+        kc = torch.zeros((n_jobs, L, sh.C, Hkv, sh.d * bits // 8), dtype=torch.uint8, device=DEV)
+        vc = torch.zeros_like(kc)
+        km = torch.zeros((n_jobs, L, G, Hkv, sh.d, 2), dtype=torch.float32, device=DEV)
+        vm = torch.zeros((n_jobs, L, sh.C, Hkv, G, 2), dtype=torch.float32, device=DEV)
+        kd, vd = k.to(DEV), v.to(DEV)
+        skip_v = n_jobs // 2  # one job without values
+        B.kvb_quantize_chunks(ctx, [dict(k=kd[i], k_codes=kc[i], k_meta=km[i], bits=bits, **({} if i == skip_v and n_jobs > 1 else
+                                    dict(v=vd[i], v_codes=vc[i], v_meta=vm[i]))) for i in range(n_jobs)])
+        B.kvb_last_status(ctx)
+        kg = k.view(n_jobs, L, G, sh.C // G, Hkv, sh.d).permute(0, 1, 2, 4, 5, 3)  # tokens of a group last
+        codes, s, mn = _eq6(kg, bits)
+        codes = codes.permute(0, 1, 2, 5, 3, 4).reshape(n_jobs, L, sh.C, Hkv, sh.d).to(torch.uint8)
+        vcodes, vs, vmn = _eq6(v.view(n_jobs, L, sh.C, Hkv, G, sh.d // G), bits)
+        vcodes = vcodes.reshape(n_jobs, L, sh.C, Hkv, sh.d).to(torch.uint8)
+        if bits == 4:
+            codes, vcodes = codes[..., 0::2] | (codes[..., 1::2] << 4), vcodes[..., 0::2] | (vcodes[..., 1::2] << 4)
+        if n_jobs > 1:
+            vcodes[skip_v], vs[skip_v], vmn[skip_v] = 0, 0, 0
+        assert torch.equal(kc.cpu(), codes)
+        assert torch.equal(km.cpu(), torch.stack([s[..., 0], mn[..., 0]], -1))
+        assert torch.equal(vc.cpu(), vcodes)
+        assert torch.equal(vm.cpu(), torch.stack([vs[..., 0], vmn[..., 0]], -1))
+    finally:
+        B.kvb_destroy(ctx)

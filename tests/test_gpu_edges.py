@@ -410,3 +410,30 @@ def test_attention_cta_pair_form_matches_oracle(option):
             assert not out[i][:, n:].any()
     finally:
         B.kvb_destroy(ctx)
+
+
+@pytest.mark.parametrize("kv_dtype,Hkv", [("bf16", 1), ("fp16", 2), ("bf16", 16)])
+@pytest.mark.parametrize("which", [1, 2, 3])
+@pytest.mark.parametrize("T", [1, 63, 64, 65, 200])
+def test_deviation_kernel_sides_and_ragged_tiles(kv_dtype, Hkv, which, T):
+    """Every form of the deviation kernel (keys, values, both) on tiles of 64 positions that are full, one short, one
+    over, and on a single position.  Bound: float32 sums of 128 squares and two hardware reciprocals, 1e-5 as stated
+    for the deviation everywhere else."""
+    sh = synth.Shape(L=3, Hq=Hkv, Hkv=Hkv, kv_dtype=kv_dtype)
+    g = torch.Generator().manual_seed(T + 10 * which)
+    a = torch.randn((sh.L, 2, T, Hkv, sh.d), generator=g)
+    b = a + 0.3 * torch.rand((sh.L, 2, T, Hkv, 1), generator=g) * torch.randn(a.shape, generator=g)
+    b[0, :, 0] = 0  # a zero row: cos 0
+    b[1, :, T - 1] = a[1, :, T - 1]
+    a, b = a.to(sh.torch_dtype), b.to(sh.torch_dtype)
+    delta = torch.full((T + 1,), 7.0, device=DEV)
+    model = B.kvb_model_desc(sh.L, sh.Hq, sh.Hkv, sh.d, sh.C, B.KVB_DT_BF16 if kv_dtype == "bf16" else B.KVB_DT_F16, sh.int4_group, 0, sh.theta)
+    assert B.kvb_deviation_static(0, model, a.to(DEV), b.to(DEV), T, which, delta[:T]) == B.KVB_OK
+    torch.cuda.synchronize()
+    x, y = a.double(), b.double()
+    cos = (x * y).sum(-1) / (x.norm(dim=-1) * y.norm(dim=-1)).clamp_min(1e-300)
+    cos[(x == y).all(-1)] = 1.0
+    sides = [s for s in (0, 1) if which >> s & 1]
+    want = 1.0 - cos[:, sides].mean(dim=(0, 1, 3))
+    assert float((delta[:T].cpu().double() - want).abs().max()) <= 1e-5
+    assert float(delta[T]) == 7.0

@@ -472,7 +472,7 @@ int kvb_assemble(kvb_ctx* c, const kvb_request* reqs, int n_req, void* cuda_stre
     c->launches += 1;
   }
   KVB_CUDA(c, launch_assemble(cd_dev, n_chunks, c->cs_table, c->dims, smem, c->status_dev, 0, nullptr,
-                              want_importance ? c->norm_sums : nullptr, c->pdl, st));
+                              want_importance ? c->norm_sums : nullptr, c->n_sm, c->pdl, st));
   c->launches += 1;
   if (want_importance) {
     KVB_CUDA(c, launch_importance_finalize(cd_dev, n_chunks, c->dims, c->norm_sums, st));
@@ -558,7 +558,7 @@ int kvb_assemble_select(kvb_ctx* c, const kvb_request* reqs, int n_req, const kv
   }
   c->acc_dirty = true;  // cleared again once both kernels are in the stream
   KVB_CUDA(c, launch_assemble(cd_dev, n_chunks, c->cs_table, c->dims, smem, c->status_dev, p->which, c->acc,
-                              want_importance ? c->norm_sums : nullptr, c->pdl, st));
+                              want_importance ? c->norm_sums : nullptr, c->n_sm, c->pdl, st));
   KVB_CUDA(c, launch_topk(rd_dev, n_req, sw_dev, c->dims, n_deviation_terms(c, p->which), ext.max_T, ext.max_k, c->acc,
                           c->status_dev, c->pdl, st));
   c->acc_dirty = false;

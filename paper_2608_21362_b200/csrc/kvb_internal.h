@@ -90,7 +90,7 @@ cudaError_t launch_rope_table(const ChunkDesc* chunks, int n_chunks, const doubl
                               float2* cs_table, cudaStream_t st);
 cudaError_t launch_assemble(const ChunkDesc* chunks, int n_chunks, const float2* cs_table, const ModelDims& m,
                             size_t smem_bytes, uint32_t* status, int which, unsigned long long* acc, double* norm_sums,
-                            bool pdl, cudaStream_t st);
+                            int n_sm, bool pdl, cudaStream_t st);
 int assemble_parts_per_layer(int Hkv);
 cudaError_t launch_importance_finalize(const ChunkDesc* chunks, int n_chunks, const ModelDims& m, const double* norm_sums,
                                        cudaStream_t st);

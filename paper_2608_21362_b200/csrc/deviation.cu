@@ -17,9 +17,13 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "deviation_math.cuh"
 #include "f32x2.cuh"
 #include "kvb_internal.h"
+#include "pdl.cuh"
+#include "table_arg.cuh"
 
 namespace kvb {
 namespace {
@@ -28,9 +32,11 @@ constexpr int kThreads = 256;
 constexpr int kTileTokens = 64;
 
 // grid (tiles over all requests, L).  A tile is kTileTokens consecutive positions of one request.
-template <int DT, int WHICH>
+template <int DT, int WHICH, typename Tab>
 __global__ void __launch_bounds__(kThreads)
-    deviation_kernel(const ReqDesc* __restrict__ reqs, int n_req, ModelDims m, unsigned long long* __restrict__ acc) {
+    deviation_kernel(const __grid_constant__ Tab table, int n_req, ModelDims m, unsigned long long* __restrict__ acc) {
+  pdl_wait();  // the table, the buffer and the cleared sums may come from the kernels before this one
+  const ReqDesc* const reqs = reinterpret_cast<const ReqDesc*>(table.base());
   // request of this tile: last r with tile_offset <= tile
   const int tile = blockIdx.x;
   int lo = 0, hi = n_req - 1;
@@ -95,15 +101,16 @@ __global__ void __launch_bounds__(kThreads)
 
 int deviation_tile_tokens() { return kTileTokens; }
 
-cudaError_t launch_deviation(const ReqDesc* reqs, int n_req, int total_tiles, const ModelDims& m, int which,
-                             unsigned long long* acc, cudaStream_t st) {
-  dim3 grid((unsigned)total_tiles, (unsigned)m.L);
-  auto launch = [&](auto kernel) { kernel<<<grid, kThreads, 0, st>>>(reqs, n_req, m, acc); };
-  if (m.dtype == KVB_DT_BF16)
-    which == 1 ? launch(deviation_kernel<KVB_DT_BF16, 1>) : which == 2 ? launch(deviation_kernel<KVB_DT_BF16, 2>) : launch(deviation_kernel<KVB_DT_BF16, 3>);
-  else
-    which == 1 ? launch(deviation_kernel<KVB_DT_F16, 1>) : which == 2 ? launch(deviation_kernel<KVB_DT_F16, 2>) : launch(deviation_kernel<KVB_DT_F16, 3>);
-  return cudaGetLastError();
+cudaError_t launch_deviation(const Table& table, int n_req, int total_tiles, const ModelDims& m, int which,
+                             unsigned long long* acc, bool pdl, cudaStream_t st) {
+  const dim3 grid((unsigned)total_tiles, (unsigned)m.L), block(kThreads);
+  return with_table(table, [&](const auto& tab) {
+    using Tab = std::decay_t<decltype(tab)>;
+    auto launch = [&](auto kernel) { return launch_pdl(pdl, kernel, grid, block, 0, st, tab, n_req, m, acc); };
+    if (m.dtype == KVB_DT_BF16)
+      return which == 1 ? launch(deviation_kernel<KVB_DT_BF16, 1, Tab>) : which == 2 ? launch(deviation_kernel<KVB_DT_BF16, 2, Tab>) : launch(deviation_kernel<KVB_DT_BF16, 3, Tab>);
+    return which == 1 ? launch(deviation_kernel<KVB_DT_F16, 1, Tab>) : which == 2 ? launch(deviation_kernel<KVB_DT_F16, 2, Tab>) : launch(deviation_kernel<KVB_DT_F16, 3, Tab>);
+  });
 }
 
 }  // namespace kvb

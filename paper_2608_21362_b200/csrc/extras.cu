@@ -6,9 +6,12 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "f32x2.cuh"
 #include "kvb_internal.h"
 #include "pdl.cuh"
+#include "table_arg.cuh"
 
 namespace kvb {
 namespace {
@@ -85,13 +88,14 @@ __device__ __forceinline__ int request_of(const ReqDesc* __restrict__ reqs, int 
 // Eq. 7, first step: a CTA per (chunk, layer) adds up the L2 norms of the chunk-layer's (token, head)
 // key rows in a fixed order -- a half-warp per 256-byte row, four rows in flight, the half-warps'
 // double-precision sums combined in warp order -- into part[chunk][layer].
-template <int DT>
+template <int DT, typename Tab>
 __global__ void __launch_bounds__(kThreads)
-    importance_kernel(const ReqDesc* __restrict__ reqs, int n_req, ModelDims m, double* __restrict__ part) {
+    importance_kernel(const __grid_constant__ Tab table, int n_req, ModelDims m, double* __restrict__ part) {
   constexpr int kUnroll = 4;
   __shared__ double s_part[kThreads / 32];
   const int item = blockIdx.x, l = blockIdx.y;
   pdl_wait();  // the table and the buffer come from the kernels before this one
+  const ReqDesc* const reqs = reinterpret_cast<const ReqDesc*>(table.base());
   const ReqDesc rq = reqs[request_of(reqs, n_req, item)];
   const int chunk = item - rq.tile_offset;
   const int H = m.Hkv, C = m.C;
@@ -140,11 +144,13 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 // Second step: a thread per chunk adds the layers' sums in layer order and takes the mean.
-__global__ void importance_mean_kernel(const ReqDesc* __restrict__ reqs, int n_req, int total_chunks, ModelDims m,
+template <typename Tab>
+__global__ void importance_mean_kernel(const __grid_constant__ Tab table, int n_req, int total_chunks, ModelDims m,
                                        const double* __restrict__ part) {
   const int item = blockIdx.x * blockDim.x + threadIdx.x;
   pdl_wait();
   if (item >= total_chunks) return;
+  const ReqDesc* const reqs = reinterpret_cast<const ReqDesc*>(table.base());
   const ReqDesc rq = reqs[request_of(reqs, n_req, item)];
   double tot = 0.0;
   for (int l = 0; l < m.L; ++l) tot += part[(size_t)item * m.L + l];
@@ -161,13 +167,16 @@ cudaError_t launch_patch_table(const PatchDesc* table, int n_req, int n_sm, cons
   return launch_pdl(pdl, patch_table_kernel, dim3((unsigned)(n_sm * kPatchCtasPerSm)), dim3(kThreads), 0, st, table, n_req, m);
 }
 
-cudaError_t launch_importance(const ReqDesc* reqs, int n_req, int total_chunks, const ModelDims& m, double* part, bool pdl, cudaStream_t st) {
+cudaError_t launch_importance(const Table& table, int n_req, int total_chunks, const ModelDims& m, double* part, bool pdl, cudaStream_t st) {
   const dim3 grid((unsigned)total_chunks, (unsigned)m.L);
-  cudaError_t e = m.dtype == KVB_DT_BF16 ? launch_pdl(pdl, importance_kernel<KVB_DT_BF16>, grid, dim3(kThreads), 0, st, reqs, n_req, m, part)
-                                         : launch_pdl(pdl, importance_kernel<KVB_DT_F16>, grid, dim3(kThreads), 0, st, reqs, n_req, m, part);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(pdl, importance_mean_kernel, dim3((unsigned)((total_chunks + 127) / 128)), dim3(128), 0, st, reqs, n_req, total_chunks, m,
-                    static_cast<const double*>(part));
+  return with_table(table, [&](const auto& tab) {
+    using Tab = std::decay_t<decltype(tab)>;
+    const cudaError_t e = m.dtype == KVB_DT_BF16 ? launch_pdl(pdl, importance_kernel<KVB_DT_BF16, Tab>, grid, dim3(kThreads), 0, st, tab, n_req, m, part)
+                                                 : launch_pdl(pdl, importance_kernel<KVB_DT_F16, Tab>, grid, dim3(kThreads), 0, st, tab, n_req, m, part);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(pdl, importance_mean_kernel<Tab>, dim3((unsigned)((total_chunks + 127) / 128)), dim3(128), 0, st, tab, n_req, total_chunks, m,
+                      static_cast<const double*>(part));
+  });
 }
 
 }  // namespace kvb

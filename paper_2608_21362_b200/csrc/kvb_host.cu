@@ -102,6 +102,18 @@ int upload(kvb_ctx* c, int slot, const uint8_t* host, size_t bytes, cudaStream_t
   return KVB_OK;
 }
 
+// Where the call's packed tables reach its kernels: by value in their arguments (the launches read the host bytes before
+// they return, so the staging slot is free again at once), or beyond kDescBlobBytes in the arena.
+int place(kvb_ctx* c, int slot, const uint8_t* host, size_t bytes, cudaStream_t st, Table* table) {
+  *table = Table{host, bytes, nullptr};
+  if (bytes <= kDescBlobBytes && !c->force_copy) {
+    c->slot_used[slot] = false;
+    return KVB_OK;
+  }
+  table->dev = c->arena_dev;
+  return upload(c, slot, host, bytes, st);
+}
+
 // Checks one request's table: chunks in prompt order tiling [0, T) exactly, enums and pointers sane.
 // need_fresh: the call reads the request's fresh tensor (the attention and the importance score do not).
 int check_request(kvb_ctx* c, const kvb_request& r, int ri, bool need_payload, bool need_fresh) {
@@ -504,15 +516,13 @@ int kvb_deviation_topk(kvb_ctx* c, const kvb_request* reqs, int n_req, const kvb
   if (st2 != KVB_OK) return st2;
   const int st3 = clear_acc_if_dirty(c, st);
   if (st3 != KVB_OK) return st3;
-  const int up = upload(c, slot, host, sizeof(ReqDesc) * (size_t)n_req + sizeof(SeamWindow) * (size_t)ext.n_seams, st);
+  Table table;
+  const int up = place(c, slot, host, sizeof(ReqDesc) * (size_t)n_req + sizeof(SeamWindow) * (size_t)ext.n_seams, st, &table);
   if (up != KVB_OK) return up;
   c->last_stream = st;
-  const ReqDesc* rd_dev = reinterpret_cast<const ReqDesc*>(c->arena_dev);
-  const SeamWindow* sw_dev = reinterpret_cast<const SeamWindow*>(c->arena_dev + sizeof(ReqDesc) * (size_t)n_req);
   c->acc_dirty = true;  // cleared again once both kernels are in the stream
-  KVB_CUDA(c, launch_deviation(rd_dev, n_req, ext.tiles, c->dims, p->which, c->acc, st));
-  KVB_CUDA(c, launch_topk(rd_dev, n_req, sw_dev, c->dims, n_deviation_terms(c, p->which), ext.max_T, ext.max_k, c->acc,
-                          c->status_dev, c->pdl, st));
+  KVB_CUDA(c, launch_deviation(table, n_req, ext.tiles, c->dims, p->which, c->acc, c->pdl, st));
+  KVB_CUDA(c, launch_topk(table, n_req, c->dims, n_deviation_terms(c, p->which), ext.max_T, ext.max_k, c->acc, c->status_dev, c->pdl, st));
   c->acc_dirty = false;
   c->launches += 2;
   return KVB_OK;
@@ -550,8 +560,6 @@ int kvb_assemble_select(kvb_ctx* c, const kvb_request* reqs, int n_req, const kv
   if (up != KVB_OK) return up;
   c->last_stream = st;
   const ChunkDesc* cd_dev = reinterpret_cast<const ChunkDesc*>(c->arena_dev);
-  const ReqDesc* rd_dev = reinterpret_cast<const ReqDesc*>(c->arena_dev + rd_off);
-  const SeamWindow* sw_dev = reinterpret_cast<const SeamWindow*>(c->arena_dev + sw_off);
   if (!rope_done) {
     KVB_CUDA(c, launch_rope_table(cd_dev, n_chunks, c->inv_freq, c->model.d / 2, c->cs_table, st));
     c->launches += 1;
@@ -559,8 +567,8 @@ int kvb_assemble_select(kvb_ctx* c, const kvb_request* reqs, int n_req, const kv
   c->acc_dirty = true;  // cleared again once both kernels are in the stream
   KVB_CUDA(c, launch_assemble(cd_dev, n_chunks, c->cs_table, c->dims, smem, c->status_dev, p->which, c->acc,
                               want_importance ? c->norm_sums : nullptr, c->n_sm, c->pdl, st));
-  KVB_CUDA(c, launch_topk(rd_dev, n_req, sw_dev, c->dims, n_deviation_terms(c, p->which), ext.max_T, ext.max_k, c->acc,
-                          c->status_dev, c->pdl, st));
+  KVB_CUDA(c, launch_topk(Table{nullptr, 0, c->arena_dev + rd_off}, n_req, c->dims, n_deviation_terms(c, p->which), ext.max_T, ext.max_k,
+                          c->acc, c->status_dev, c->pdl, st));
   c->acc_dirty = false;
   c->launches += 2;
   if (want_importance) {  // after the selection, so the dependent-launch chain stitch -> selection stays as it is
@@ -704,10 +712,11 @@ int kvb_chunk_importance(kvb_ctx* c, const kvb_request* reqs, int n_req, float* 
     rd[r] = d;
     chunks += reqs[r].n_chunks;
   }
-  const int up = upload(c, slot, host, sizeof(ReqDesc) * (size_t)n_req, st);
+  Table table;
+  const int up = place(c, slot, host, sizeof(ReqDesc) * (size_t)n_req, st, &table);
   if (up != KVB_OK) return up;
   c->last_stream = st;
-  KVB_CUDA(c, launch_importance(reinterpret_cast<const ReqDesc*>(c->arena_dev), n_req, chunks, c->dims, c->norm_sums, c->pdl, st));
+  KVB_CUDA(c, launch_importance(table, n_req, chunks, c->dims, c->norm_sums, c->pdl, st));
   c->launches += 2;
   return KVB_OK;
 }

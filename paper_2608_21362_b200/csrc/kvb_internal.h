@@ -81,6 +81,13 @@ struct ModelDims {
 // cs_table[n_rope_chunks][half_d] from their delta_pos.
 constexpr size_t kDescBlobSmall = 3840;
 constexpr size_t kDescBlobBytes = 16384;
+// A call's packed tables (csrc/table_arg.cuh): `bytes` bytes at `host`, read before the launch returns, or, dev != NULL,
+// already in device memory.
+struct Table {
+  const void* host;
+  size_t bytes;
+  const uint8_t* dev;
+};
 cudaError_t launch_store_blob(const void* host_bytes, size_t bytes, uint8_t* dst, int n_rope_chunks, const double* inv_freq,
                               int half_d, float2* cs_table, bool pdl, cudaStream_t st);
 // launch_assemble: acc != NULL fuses the deviation sums (which: bit 0 keys, bit 1 values) into the stitch;
@@ -97,12 +104,14 @@ cudaError_t launch_importance_finalize(const ChunkDesc* chunks, int n_chunks, co
 size_t assemble_smem_bytes(const ModelDims& m, int mode);
 cudaError_t assemble_configure(size_t max_smem);
 
-cudaError_t launch_deviation(const ReqDesc* reqs, int n_req, int total_tiles, const ModelDims& m, int which,
-                             unsigned long long* acc, cudaStream_t st);
+// request descriptors at the start of the table
+cudaError_t launch_deviation(const Table& table, int n_req, int total_tiles, const ModelDims& m, int which,
+                             unsigned long long* acc, bool pdl, cudaStream_t st);
 int deviation_tile_tokens();
 
-cudaError_t launch_topk(const ReqDesc* reqs, int n_req, const SeamWindow* seams, const ModelDims& m, int n_terms,
-                        int max_T, int max_k, unsigned long long* acc, uint32_t* status, bool pdl, cudaStream_t st);
+// request descriptors at the start of the table, then the window list
+cudaError_t launch_topk(const Table& table, int n_req, const ModelDims& m, int n_terms, int max_T, int max_k, unsigned long long* acc,
+                        uint32_t* status, bool pdl, cudaStream_t st);
 cudaError_t topk_configure();
 int topk_max_T();
 int topk_max_k();
@@ -132,7 +141,7 @@ cudaError_t launch_attention_pair(const ReqDesc* reqs, const void* maps, int n_r
 cudaError_t launch_patch_inline(const PatchInline& descs, int n_req, int n_sm, const ModelDims& m, bool pdl, cudaStream_t st);
 cudaError_t launch_patch_table(const PatchDesc* table, int n_req, int n_sm, const ModelDims& m, bool pdl, cudaStream_t st);
 // part: [total_chunks][L] doubles of scratch (the per-layer sums); two launches
-cudaError_t launch_importance(const ReqDesc* reqs, int n_req, int total_chunks, const ModelDims& m, double* part, bool pdl, cudaStream_t st);
+cudaError_t launch_importance(const Table& table, int n_req, int total_chunks, const ModelDims& m, double* part, bool pdl, cudaStream_t st);
 
 // One chunk to quantise (device memory).  k / v NULL: that side is not wanted.
 struct QuantJob {

@@ -19,8 +19,11 @@
 // shared-memory access.
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "kvb_internal.h"
 #include "pdl.cuh"
+#include "table_arg.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -124,8 +127,9 @@ __device__ __forceinline__ uint32_t rank_by_runs(unsigned long long& v, int n, i
 // One CTA per request: the form for prompts of up to kSingleTokens positions, where a cluster's
 // barriers would cost more than its CTAs save.  Steps as in the cluster kernel below, except that the
 // k winners are sorted by a bitonic network (one element per thread, in a register).
+template <typename Tab>
 __global__ void __launch_bounds__(kThreads, 1)
-    topk_single_kernel(const ReqDesc* __restrict__ reqs, const SeamWindow* __restrict__ seams, float inv_scale,
+    topk_single_kernel(const __grid_constant__ Tab table, int n_req, float inv_scale,
                 unsigned long long* __restrict__ acc, int t_pad, uint32_t* __restrict__ status) {
   extern __shared__ __align__(16) uint8_t smem[];
   uint32_t* s_keys = reinterpret_cast<uint32_t*>(smem);                                   // [t_pad]
@@ -138,6 +142,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ uint32_t s_pick[2];       // chosen bin, remaining need
 
   pdl_wait();  // descriptors and deviation sums come from the kernels before this one
+  const ReqDesc* const reqs = reinterpret_cast<const ReqDesc*>(table.base());
+  const SeamWindow* const seams = reinterpret_cast<const SeamWindow*>(reqs + n_req);
   const ReqDesc rq = reqs[blockIdx.x];
   const int T = rq.T, k = min(rq.k, T);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -369,8 +375,9 @@ struct Shared {
   uint32_t n_union;       // selected positions of the slice after the union with the windows
 };
 
+template <typename Tab>
 __global__ void __launch_bounds__(kThreads, 1)
-    topk_cluster_kernel(const ReqDesc* __restrict__ reqs, const SeamWindow* __restrict__ seams, float inv_scale,
+    topk_cluster_kernel(const __grid_constant__ Tab table, int n_req, float inv_scale,
                         unsigned long long* __restrict__ acc, int slice_pad, int k_pad, uint32_t* __restrict__ status) {
   extern __shared__ __align__(16) uint8_t smem[];
   // dynamic: keys of the slice; inverted keys and positions of the slice's winners (index order);
@@ -401,6 +408,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (clustered) cluster.sync(); else __syncthreads();
   };
   pdl_wait();  // descriptors and deviation sums come from the kernels before this one
+  const ReqDesc* const reqs = reinterpret_cast<const ReqDesc*>(table.base());
+  const SeamWindow* const seams = reinterpret_cast<const SeamWindow*>(reqs + n_req);
   const ReqDesc rq = reqs[blockIdx.x / S];
   const int T = rq.T, k = min(rq.k, T);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -755,13 +764,20 @@ int topk_max_T() { return kMaxT; }
 int topk_max_k() { return kMaxK; }
 
 cudaError_t topk_configure() {
-  cudaError_t e = cudaFuncSetAttribute(topk_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster_smem(kMaxSlice, kMaxK));
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(topk_single_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)single_smem(kSingleTokens, kSingleTokens));
+  auto one = [](auto tab) {
+    using Tab = decltype(tab);
+    const cudaError_t e = cudaFuncSetAttribute(topk_cluster_kernel<Tab>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster_smem(kMaxSlice, kMaxK));
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(topk_single_kernel<Tab>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)single_smem(kSingleTokens, kSingleTokens));
+  };
+  cudaError_t e = one(TableAddress{});
+  if (e == cudaSuccess) e = one(TableBytes<kDescBlobSmall>{});
+  if (e == cudaSuccess) e = one(TableBytes<kDescBlobBytes>{});
+  return e;
 }
 
-cudaError_t launch_topk(const ReqDesc* reqs, int n_req, const SeamWindow* seams, const ModelDims& m, int n_terms,
-                        int max_T, int max_k, unsigned long long* acc, uint32_t* status, bool pdl, cudaStream_t st) {
+cudaError_t launch_topk(const Table& table, int n_req, const ModelDims& m, int n_terms, int max_T, int max_k, unsigned long long* acc,
+                        uint32_t* status, bool pdl, cudaStream_t st) {
   (void)m;
   const int S = cluster_size(max_T);
   const float inv_scale = (float)(1.0 / (1099511627776.0 * (double)n_terms));  // 2^-40 / n_terms
@@ -783,12 +799,16 @@ cudaError_t launch_topk(const ReqDesc* reqs, int n_req, const SeamWindow* seams,
     int k_pow2 = 1;
     while (k_pow2 < max_k) k_pow2 <<= 1;
     cfg.dynamicSmemBytes = single_smem(t_pad, k_pow2);
-    return cudaLaunchKernelEx(&cfg, topk_single_kernel, reqs, seams, inv_scale, acc, t_pad, status);
+    return with_table(table, [&](const auto& tab) {
+      return cudaLaunchKernelEx(&cfg, topk_single_kernel<std::decay_t<decltype(tab)>>, tab, n_req, inv_scale, acc, t_pad, status);
+    });
   }
   const int slice_pad = ((max_T + 32 * S - 1) / (32 * S)) * 32;  // the largest slice of the batch
   const int k_pad = ((max_k < 1 ? 1 : max_k) + 3) & ~3;
   cfg.dynamicSmemBytes = cluster_smem(slice_pad, k_pad);
-  return cudaLaunchKernelEx(&cfg, topk_cluster_kernel, reqs, seams, inv_scale, acc, slice_pad, k_pad, status);
+  return with_table(table, [&](const auto& tab) {
+    return cudaLaunchKernelEx(&cfg, topk_cluster_kernel<std::decay_t<decltype(tab)>>, tab, n_req, inv_scale, acc, slice_pad, k_pad, status);
+  });
 }
 
 }  // namespace kvb

@@ -437,3 +437,38 @@ def test_deviation_kernel_sides_and_ragged_tiles(kv_dtype, Hkv, which, T):
     want = 1.0 - cos[:, sides].mean(dim=(0, 1, 3))
     assert float((delta[:T].cpu().double() - want).abs().max()) <= 1e-5
     assert float(delta[T]) == 7.0
+
+
+@pytest.mark.parametrize("n_req", [1, 31, 40, 41, 171])
+def test_tables_of_every_size_reach_the_selection_and_the_importance(n_req):
+    """Request tables of both by-value argument sizes (up to 3840 and 16384 bytes) and of the copy beyond them, at the
+    edges: kvb_deviation_topk and kvb_chunk_importance give what one request at a time gives, bit for bit."""
+    sh = synth.Shape(L=2)
+    n_chunks = [1 + i % 3 for i in range(n_req)]
+    g = torch.Generator().manual_seed(n_req)
+    reqs = []
+    for n in n_chunks:
+        plan = synth._request(n * sh.C, sh.C, [synth.MODE_FP16 if i % 2 else synth.MODE_FRESH for i in range(n)], [i * sh.C for i in range(n)])
+        kv = torch.randn((sh.L, 2, n * sh.C, sh.Hkv, sh.d), generator=g).to(sh.torch_dtype).to(DEV)
+        fresh = (kv.float() + 0.1 * torch.randn(kv.shape, generator=g).to(DEV)).to(sh.torch_dtype)
+        reqs.append(synth.Request(plan, [synth.Chunk(c) for c in plan.chunks], fresh, kv, None, 0))
+    Ts = [r.plan.T for r in reqs]
+    ks = [B.kvb_select_count(t, 0.15) for t in Ts]
+    ctx = B.create_for_shape(sh, 0, max_requests=256, max_chunks_total=512)
+    try:
+        def run(rs, ts, kk):
+            tbl, sel = B.RequestTable(rs), B.SelectionTable(ts, kk, ts, DEV)
+            B.kvb_deviation_topk(ctx, tbl, 0.15, -1, 16, 0, 3, sel, sink_tokens=2)
+            imp = [torch.zeros(t // sh.C, device=DEV) for t in ts]
+            B.kvb_chunk_importance(ctx, tbl, imp)
+            B.kvb_last_status(ctx)
+            return sel, imp
+
+        sel, imp = run(reqs, Ts, ks)
+        for i in sorted({0, 1 % n_req, n_req // 2, n_req - 1}):
+            one, one_imp = run([reqs[i]], [Ts[i]], [ks[i]])
+            assert int(sel.n_sel[i]) == int(one.n_sel[0]) > 0
+            for a, b in ((sel.delta[i], one.delta[0]), (sel.rank[i], one.rank[0]), (sel.sel[i], one.sel[0]), (imp[i], one_imp[0])):
+                assert torch.equal(a, b)
+    finally:
+        B.kvb_destroy(ctx)

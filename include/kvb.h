@@ -327,6 +327,12 @@ int64_t kvb_launch_count(kvb_ctx* ctx);
  *                                 neighbouring tiles per CTA that share every K/V
  *                                 sub-block in shared memory, one CTA per SM; same
  *                                 result to the attention tolerance
+ *   "quantize_stalled_fetch"      default 0; 1 makes the part of the quantiser that fetches
+ *                                 its tiles stop early (a different number of tiles into
+ *                                 every CTA), as if its loads never landed, and shortens
+ *                                 the waits: the error path of a stuck wait.  A chunk side
+ *                                 is then left unwritten in part, nothing else is written,
+ *                                 and kvb_last_status reports 0x1
  * The first three settings compute the same bits; the tests compare them.
  * Unknown key or value: KVB_ERR_INVALID_ARG. */
 int kvb_set_debug_option(kvb_ctx* ctx, const char* key, int value);

@@ -45,6 +45,7 @@ struct kvb_ctx {
   bool pdl = true;             // programmatic dependent launch along the kernel chain
   bool attn_pair = false;      // attention on CTA pairs (tcgen05 cta_group::2) instead of single CTAs
   bool attn_dual = false;      // attention with two tiles per CTA sharing K/V, one CTA per SM
+  bool quant_stalled = false;  // the quantiser's fetching warps stop before they are through (its waits' error path)
   cudaStream_t last_stream = nullptr;
   int64_t launches = 0;
   char err[512] = {0};
@@ -295,6 +296,7 @@ int kvb_set_debug_option(kvb_ctx* c, const char* key, int value) {
   else if (strcmp(key, "attention_one_tile_per_cta") == 0) c->attn_one_tile = value != 0;
   else if (strcmp(key, "attention_cta_pairs") == 0) c->attn_pair = value != 0;
   else if (strcmp(key, "attention_two_tiles") == 0) c->attn_dual = value != 0;
+  else if (strcmp(key, "quantize_stalled_fetch") == 0) c->quant_stalled = value != 0;
   else return fail(c, KVB_ERR_INVALID_ARG, "unknown debug option '%s'", key);
   return KVB_OK;
 }
@@ -750,7 +752,7 @@ int kvb_quantize_chunks(kvb_ctx* c, const kvb_quantize_job* jobs, int n_jobs, vo
     QuantJob qj[kQuantInline];
     fill(qj);
     c->last_stream = st;
-    KVB_CUDA(c, launch_quantize_inline(qj, n_jobs, c->dims, c->inv_freq, c->status_dev, c->n_sm, c->pdl, st));
+    KVB_CUDA(c, launch_quantize_inline(qj, n_jobs, c->dims, c->inv_freq, c->status_dev, c->n_sm, c->pdl, c->quant_stalled, st));
   } else {
     uint8_t* host = nullptr;
     const int slot_code = take_slot(c, &host);
@@ -760,7 +762,7 @@ int kvb_quantize_chunks(kvb_ctx* c, const kvb_quantize_job* jobs, int n_jobs, vo
     const int up = upload(c, slot, host, sizeof(QuantJob) * (size_t)n_jobs, st);
     if (up != KVB_OK) return up;
     c->last_stream = st;
-    KVB_CUDA(c, launch_quantize_table(reinterpret_cast<const QuantJob*>(c->arena_dev), n_jobs, c->dims, c->inv_freq, c->status_dev, c->n_sm, c->pdl, st));
+    KVB_CUDA(c, launch_quantize_table(reinterpret_cast<const QuantJob*>(c->arena_dev), n_jobs, c->dims, c->inv_freq, c->status_dev, c->n_sm, c->pdl, c->quant_stalled, st));
   }
   c->launches += 1;
   return KVB_OK;

@@ -157,11 +157,12 @@ struct QuantJob {
   int32_t reserved;
 };
 // Up to kQuantInline jobs travel as the kernel's own argument (host_jobs is read before the call returns),
-// more through a table in device memory.  inv_freq: [d/2] doubles, device.
+// more through a table in device memory.  inv_freq: [d/2] doubles, device.  stalled: the fetching warps stop before they
+// are through and the waits are short (option quantize_stalled_fetch).
 constexpr int kQuantInline = (int)(kDescBlobBytes / sizeof(QuantJob));
-cudaError_t launch_quantize_inline(const QuantJob* host_jobs, int n_jobs, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl,
+cudaError_t launch_quantize_inline(const QuantJob* host_jobs, int n_jobs, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl, bool stalled,
                                    cudaStream_t st);
-cudaError_t launch_quantize_table(const QuantJob* table, int n_jobs, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl,
+cudaError_t launch_quantize_table(const QuantJob* table, int n_jobs, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl, bool stalled,
                                   cudaStream_t st);
 cudaError_t quantize_configure();
 

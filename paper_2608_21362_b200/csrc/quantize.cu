@@ -46,7 +46,8 @@ constexpr int kRows = 128;     // rows of a tile: the tokens of a chunk, or that
 constexpr int kD = 128;        // head_dim
 constexpr int kRowsPerWarp = kRows / kWarps;
 constexpr uint32_t kTileBytes = kRows * kD * 2;
-constexpr uint32_t kWaitLimit = 1u << 22;
+constexpr uint32_t kWaitLimit = 1u << 22;         // polls after which a wait gives up
+constexpr uint32_t kStalledWaitLimit = 1u << 10;  // the same in a launch whose fetching warps are made to stop (option quantize_stalled_fetch)
 constexpr int kStages = 5;     // tile buffers: one in work per group, the others in flight
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -68,11 +69,36 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Bounded wait: gives up after kWaitLimit polls (never expected; keeps a bad launch from hanging).
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-  for (uint32_t i = 0; i < kWaitLimit; ++i) {
-    if (mbar_try_wait(bar, parity)) return true;
+// Bounded wait of a whole warp: gives up after `limit` polls (never expected; keeps a bad launch from hanging).  Every lane
+// gets the same answer.
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32_t limit) {
+  for (uint32_t i = 0; i < limit; ++i) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
     if (i > 64) __nanosleep(64);
+  }
+  return false;
+}
+// a group's own barrier
+__device__ __forceinline__ void group_sync(int group) { asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(kWarps * 32) : "memory"); }
+// After a warp's wait for its group's tile has run out: true if the tile has landed after all, false if the wait has run out
+// for every warp of the group (`gave_up` counts them; kWarps is final).  So the warps of a group leave together or go on
+// together, and none is left waiting in group_sync.  It ends: a tile that one warp has seen stays until all are through with
+// it, and a warp that has not seen it gives up too.
+__device__ __noinline__ bool landed_late(uint64_t* bar, uint32_t parity, uint32_t limit, uint32_t* gave_up) {
+  const bool first = (threadIdx.x & 31) == 0;
+  uint32_t n = first ? atomicAdd(gave_up, 1u) + 1u : 0u;
+  n = __shfl_sync(0xffffffffu, n, 0);
+  for (uint32_t i = 0; i < limit && n < (uint32_t)kWarps; ++i) {
+    const bool landed = __all_sync(0xffffffffu, mbar_try_wait(bar, parity));
+    bool back = false;
+    if (first) {
+      const uint32_t seen = landed ? atomicCAS(gave_up, n, n - 1u) : *reinterpret_cast<volatile uint32_t*>(gave_up);
+      back = landed && seen == n;
+      n = seen;
+    }
+    if (__shfl_sync(0xffffffffu, back, 0)) return true;
+    n = __shfl_sync(0xffffffffu, n, 0);
+    if (!landed) __nanosleep(64);
   }
   return false;
 }
@@ -89,8 +115,6 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
 __device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
   asm volatile("cp.async.mbarrier.arrive.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-// a group's own barrier
-__device__ __forceinline__ void group_sync(int group) { asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(kWarps * 32) : "memory"); }
 
 constexpr float kMagic = 8388608.0f;  // 2^23
 // The code of a value: rint(x / s) clamped to [0, levels], x = v - mn, subtraction and division being IEEE float32.
@@ -245,13 +269,14 @@ __device__ __forceinline__ int ext_at(int w, int max, int ch) { return w * 2 * k
 template <int DT, typename Jobs>
 __global__ void __launch_bounds__(kThreads, 1)
     quantize_batch_kernel(const __grid_constant__ Jobs jobs, ModelDims m, uint32_t n_items, const double* __restrict__ inv_freq,
-                          uint32_t* __restrict__ status) {
+                          uint32_t* __restrict__ status, bool stalled) {
   extern __shared__ __align__(128) uint8_t smem[];  // kStages tiles
   __shared__ __align__(16) float s_ext_all[kGroups][kWarps * 2 * kD];  // see ext_at
   __shared__ __align__(16) float s_par_all[kGroups][3][4 * kD];        // keys: min, reciprocal and -scale of every [token group][channel]
   __shared__ float2 s_rot[kStages][kD / 2];               // cos / sin of a chunk's rotation; a ring, in use by at most kStages tiles
   __shared__ TileDesc s_tile[kStages];
   __shared__ __align__(8) uint64_t s_full[kStages], s_empty[kStages];
+  __shared__ uint32_t s_gave_up[kGroups];  // warps of the group whose wait for the tile ran out
   const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) & (kWarps - 1), group = threadIdx.x / (kWarps * 32);
   const int tid = threadIdx.x & (kWarps * 32 - 1);  // within the group
   const int H = m.Hkv, log_h = __ffs(H) - 1;
@@ -263,16 +288,22 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (threadIdx.x < kStages) {
     mbar_init(&s_full[threadIdx.x], kFetchers);
     mbar_init(&s_empty[threadIdx.x], kWarps);
+    if (threadIdx.x < kGroups) s_gave_up[threadIdx.x] = 0;
   }
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   __syncthreads();
   pdl_wait();  // inputs may come from the kernel before this one, and it may still read what this one writes
+
+  // A wait that runs out sets the status and ends the warp (a group's warps together, see landed_late): it knows neither the
+  // tile nor where its codes belong.  The fetching warps that wait for the group's buffers then run out of a wait in turn.
+  const uint32_t limit = stalled ? kStalledWaitLimit : kWaitLimit;
 
   if (group == kGroups) {
     // ------------------------------ the fetching warps: descriptors, rotation tables and copies, up to kStages tiles ahead
     Tile t(first, log_h, m.L);
     uint32_t rot_job = 0xFFFFFFFFu, stage = 0, phase = 1;  // a fresh barrier passes a wait for the phase before its first
     int rot_buf = 0;
+    uint32_t left = stalled ? blockIdx.x % (2 * kStages) : 0xFFFFFFFFu;  // tiles until a stalled fetch
     for (uint32_t item = first; item < last + kGroups; ++item, t.next(H, m.L)) {
       const bool end = item >= last;  // an end mark for every group
       const uint8_t* x = nullptr;
@@ -289,7 +320,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                             t.kv ? ((size_t)t.l * H + t.h) * kRows * G : ((size_t)t.l * G * H + t.h) * kD, jb.meta16);
         td.kv = t.kv, td.bits = jb.bits, td.meta16 = jb.meta16, td.rot = -1;
       }
-      if (!mbar_wait(&s_empty[stage], phase) && lane == 0) atomicOr(status, DEV_STATUS_WAIT_TIMEOUT);
+      if (left-- == 0) return;
+      if (!mbar_wait(&s_empty[stage], phase, limit)) {
+        if (lane == 0) atomicOr(status, DEV_STATUS_WAIT_TIMEOUT);
+        asm volatile("cp.async.wait_all;" ::: "memory");  // the copies in flight land before their buffers are given up
+        for (uint32_t i = 0; i < kStages; ++i) mbar_wait(&s_full[i], i < stage ? phase ^ 1u : phase, limit);
+        return;
+      }
       if (!end && !t.kv && job_at(jobs, t.job).unrotate_from >= 0) {
         if (rot_job != t.job) {
           rot_job = t.job;
@@ -330,7 +367,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   float (*const s_par)[4 * kD] = s_par_all[group];
   uint32_t phase = 0;
   for (uint32_t stage = group;;) {  // every kGroups-th tile
-    if (!mbar_wait(&s_full[stage], phase)) atomicOr(status, DEV_STATUS_WAIT_TIMEOUT);
+    if (!mbar_wait(&s_full[stage], phase, limit)) {
+      if (lane == 0) atomicOr(status, DEV_STATUS_WAIT_TIMEOUT);
+      if (!landed_late(&s_full[stage], phase, limit, &s_gave_up[group])) return;
+    }
     const TileDesc td = s_tile[stage];
     if (!td.codes) break;
     const uint8_t* const tile = smem + stage * kTileBytes;
@@ -616,21 +656,21 @@ cudaError_t configure_type() {
 }
 
 template <typename Jobs>
-cudaError_t launch_with(const Jobs& jobs, int n_jobs, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl, cudaStream_t st) {
+cudaError_t launch_with(const Jobs& jobs, int n_jobs, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl, bool stalled, cudaStream_t st) {
   const long long n_items = (long long)n_jobs * m.L * 2 * m.Hkv;
   if (n_items > 0xFFFFFFFFll) return cudaErrorInvalidValue;
   // one CTA per SM
   const dim3 grid((unsigned)(n_items < n_sm ? n_items : n_sm)), block(kThreads);
   if (m.dtype == KVB_DT_BF16)
-    return launch_pdl(pdl, quantize_batch_kernel<KVB_DT_BF16, Jobs>, grid, block, kSmemBytes, st, jobs, m, (uint32_t)n_items, inv_freq, status);
-  return launch_pdl(pdl, quantize_batch_kernel<KVB_DT_F16, Jobs>, grid, block, kSmemBytes, st, jobs, m, (uint32_t)n_items, inv_freq, status);
+    return launch_pdl(pdl, quantize_batch_kernel<KVB_DT_BF16, Jobs>, grid, block, kSmemBytes, st, jobs, m, (uint32_t)n_items, inv_freq, status, stalled);
+  return launch_pdl(pdl, quantize_batch_kernel<KVB_DT_F16, Jobs>, grid, block, kSmemBytes, st, jobs, m, (uint32_t)n_items, inv_freq, status, stalled);
 }
 
 template <int N>
-cudaError_t launch_inline(const QuantJob* host_jobs, int n_jobs, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl, cudaStream_t st) {
+cudaError_t launch_inline(const QuantJob* host_jobs, int n_jobs, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl, bool stalled, cudaStream_t st) {
   InlineJobs<N> jobs;
   memcpy(jobs.d, host_jobs, sizeof(QuantJob) * (size_t)n_jobs);
-  return launch_with(jobs, n_jobs, m, inv_freq, status, n_sm, pdl, st);
+  return launch_with(jobs, n_jobs, m, inv_freq, status, n_sm, pdl, stalled, st);
 }
 
 }  // namespace
@@ -640,16 +680,16 @@ cudaError_t quantize_configure() {
   return e == cudaSuccess ? configure_type<KVB_DT_F16>() : e;
 }
 
-cudaError_t launch_quantize_inline(const QuantJob* host_jobs, int n_jobs, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl,
+cudaError_t launch_quantize_inline(const QuantJob* host_jobs, int n_jobs, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl, bool stalled,
                                    cudaStream_t st) {
-  if (n_jobs <= kSmallInline) return launch_inline<kSmallInline>(host_jobs, n_jobs, m, inv_freq, status, n_sm, pdl, st);
-  if (n_jobs <= kQuantInline) return launch_inline<kQuantInline>(host_jobs, n_jobs, m, inv_freq, status, n_sm, pdl, st);
+  if (n_jobs <= kSmallInline) return launch_inline<kSmallInline>(host_jobs, n_jobs, m, inv_freq, status, n_sm, pdl, stalled, st);
+  if (n_jobs <= kQuantInline) return launch_inline<kQuantInline>(host_jobs, n_jobs, m, inv_freq, status, n_sm, pdl, stalled, st);
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_quantize_table(const QuantJob* table, int n_jobs, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl,
+cudaError_t launch_quantize_table(const QuantJob* table, int n_jobs, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl, bool stalled,
                                   cudaStream_t st) {
-  return launch_with(table, n_jobs, m, inv_freq, status, n_sm, pdl, st);
+  return launch_with(table, n_jobs, m, inv_freq, status, n_sm, pdl, stalled, st);
 }
 
 }  // namespace kvb

@@ -227,3 +227,49 @@ def test_job_counts_and_extreme_ranges(n_jobs, L, Hkv, bits):
         assert torch.equal(vm.cpu(), torch.stack([vs[..., 0], vmn[..., 0]], -1))
     finally:
         B.kvb_destroy(ctx)
+
+
+@pytest.mark.parametrize("Hkv,bits,compact", [(1, 8, False), (2, 8, True), (2, 4, False), (4, 4, True)])
+def test_quantiser_whose_loads_stop_reports_it_and_writes_nothing_else(Hkv, bits, compact):
+    """The fetching warps stop a different number of tiles into every CTA (none in some), as if the loads never landed:
+    every wait gives up, the status says so, a tile is written as a whole or not at all, and the context stays usable."""
+    sh = synth.Shape(L=36, Hq=Hkv, Hkv=Hkv)
+    n, G, pad = 8 // Hkv, 1 if bits == 8 else 4, 4096
+    mt = torch.float16 if compact else torch.float32
+    ctx = B.create_for_shape(sh, 0)
+    try:
+        g = torch.Generator(device=DEV).manual_seed(3)
+        k, v = (torch.randn((n, sh.L, sh.C, Hkv, sh.d), generator=g, device=DEV).to(sh.torch_dtype) for _ in range(2))
+        shapes = {"k_codes": (n, sh.L, sh.C, Hkv, sh.d * bits // 8), "v_codes": (n, sh.L, sh.C, Hkv, sh.d * bits // 8),
+                  "k_meta": (n, sh.L, G, Hkv, sh.d, 2 * mt.itemsize), "v_meta": (n, sh.L, sh.C, Hkv, G, 2 * mt.itemsize)}
+        size = {a: int(np.prod(s)) for a, s in shapes.items()}
+        pool = torch.empty(sum(size.values()) + pad * (len(size) + 1), dtype=torch.uint8, device=DEV)
+        guard = torch.ones(pool.numel(), dtype=torch.bool, device=DEV)
+        out, at = {}, pad
+        for a, s in shapes.items():
+            out[a] = pool[at : at + size[a]].view(s)
+            guard[at : at + size[a]] = False
+            at += size[a] + pad
+        jobs = [dict(bits=bits, unrotate_from=i - 1, meta_fp16=compact, k=k[i], v=v[i], k_codes=out["k_codes"][i], v_codes=out["v_codes"][i],
+                     k_meta=out["k_meta"][i].view(mt), v_meta=out["v_meta"][i].view(mt)) for i in range(n)]
+
+        def run(stalled):
+            pool.fill_(0xA5)
+            B.kvb_set_debug_option(ctx, "quantize_stalled_fetch", stalled)
+            B.kvb_quantize_chunks(ctx, jobs)
+            assert B.kvb_last_status(ctx, check=False) == (B.KVB_ERR_DEVICE_STATUS if stalled else B.KVB_OK)
+            assert B.kvb_last_status(ctx, check=False) == B.KVB_OK
+            assert bool((pool[guard] == 0xA5).all())
+            # a row per tile: the tokens of one head's keys, or 128 (token, head) rows of values
+            tiles = lambda a: (out[a].transpose(2, 3) if a[0] == "k" else out[a]).reshape(n * sh.L * Hkv, -1).clone()
+            return torch.cat([tiles("k_codes"), tiles("k_meta")], 1), torch.cat([tiles("v_codes"), tiles("v_meta")], 1)
+
+        want = run(0)
+        for got, whole in zip(run(1), want):
+            written = (got == whole).all(1)
+            untouched = (got == 0xA5).all(1)
+            assert bool((written | untouched).all()) and bool(written.any()) and bool(untouched.any())
+        for got, whole in zip(run(0), want):
+            assert torch.equal(got, whole)
+    finally:
+        B.kvb_destroy(ctx)

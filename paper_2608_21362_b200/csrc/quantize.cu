@@ -140,9 +140,10 @@ __device__ __noinline__ uint32_t code_exact(float v, float mn, float s, float le
   c = fminf(fmaxf(c, 0.f), levels);
   return (uint32_t)c;
 }
-// y = RN(1 / s); the rest of the reciprocal is y (1 - y s).  Where the remainders of code_pair could leave float32's normal
-// range (a group of tiny or huge range, or none that is finite) y is zero, and the IEEE division decides for the group.
-__device__ __forceinline__ float reciprocal(float s) { return s >= 1e-20f && s <= 1e20f ? __frcp_rn(s) : 0.f; }
+// y = RN(1 / s); the rest of the reciprocal is y (1 - y s).  Within 1e-30 .. 1e30 code_pair's remainder is exact for every
+// quotient that can decide (from 1/4 on it is a multiple of 2^-25 2^-23 2^-100, above float32's smallest number) and nothing
+// overflows.  Outside, or where the extremes are not finite, y is zero, and the IEEE division decides for the group.
+__device__ __forceinline__ float reciprocal(float s) { return s >= 1e-30f && s <= 1e30f ? __frcp_rn(s) : 0.f; }
 __device__ __forceinline__ float min3(float a, float b, float c) {
   float d;
   asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
@@ -265,6 +266,68 @@ struct __align__(16) TileDesc {
 // rows of a values tile.  The channels of every other warp are shifted by 16, so that a read of 16 channels of two
 // neighbouring warps hits 32 banks.
 __device__ __forceinline__ int ext_at(int w, int max, int ch) { return w * 2 * kD + max * kD + (ch ^ ((w & 1) << 4)); }
+
+// The codes of the groups outside the reciprocal's range, decided again by the division once the warp has stored the codes of
+// its part of a tile.  All lanes share the work: 16 chunks of 36 layers and 2 heads, one channel and one row of each at 1e-35,
+// take 29 (int8) and 36 us (rotated int4) against 23 and 28 with none; the lanes that own them alone took 69 and 83.
+// keys: a byte column (a channel, or a pair of 4-bit ones) of the warp's 16 tokens per half-warp
+template <int DT, int BITS, bool ROT>
+__device__ __noinline__ void redo_keys(const uint8_t* tile, const float (*par)[4 * kD], const float2* rot, uint8_t* codes, uint32_t row_stride, int warp) {
+  constexpr float levels = (float)((1 << BITS) - 1);
+  const int lane = threadIdx.x & 31, p = lane & 15, t = warp * kRowsPerWarp + p;
+  const int g0 = BITS == 8 ? 0 : warp / (kWarps / 4) * kD;  // the token group's first channel in `par`
+  uint32_t odd = 0;  // bit 4 side + e: channel 4 p + e of that side
+  for (int n = 0; n < 8; ++n) odd |= (par[1][g0 + (n >> 2) * (kD / 2) + 4 * p + (n & 3)] > 0.f ? 0u : 1u) << n;
+  if (BITS == 4) odd = (odd | odd >> 1) & 0x55u;
+  __syncwarp();  // the codes stored before come first
+  for (uint32_t who; (who = __ballot_sync(0xffffffffu, odd != 0) & 0xFFFFu) != 0;) {
+    const uint32_t more = who & (who - 1);
+    const int q0 = __ffs(who) - 1, q1 = more ? __ffs(more) - 1 : q0;  // a lane whose channels are odd for each half-warp
+    const int q = lane < 16 ? q0 : q1, n = __ffs(__shfl_sync(0xffffffffu, odd, q)) - 1;
+    if (p == q0 || p == q1) odd &= odd - 1;
+    const int side = n >> 2;
+    uint32_t w = 0;
+#pragma unroll
+    for (int e = 0; e < 8 / BITS; ++e) {
+      const int c = 4 * q + (n & 3) + e;
+      const uint8_t* const at = tile + t * (kD * 2) + 2 * c;  // the low channel; its partner 64 channels on
+      float v = value_of<DT>(at + side * kD);
+      if (ROT) v = fmaf(v, rot[c].x, __fmul_rn(value_of<DT>(at + (side ^ 1) * kD), side ? -rot[c].y : rot[c].y));  // as in `rotated`
+      const int gc = g0 + side * (kD / 2) + c;
+      w |= code_exact(v, par[0][gc], -par[2][gc], levels) << (BITS * e);
+    }
+    codes[(uint32_t)t * row_stride + (uint32_t)(side * (kD / 2) + 4 * q + (n & 3)) * BITS / 8] = (uint8_t)w;
+  }
+}
+// values: a group of a row per 32 or 8 lanes, four channels a lane.  s_row: (min, reciprocal, its rest, -scale) of [row][group]
+template <int DT, int BITS>
+__device__ __noinline__ void redo_values(const uint8_t* tile, const float4* s_row, uint8_t* codes, int warp) {
+  constexpr float levels = (float)((1 << BITS) - 1);
+  constexpr int G = BITS == 8 ? 1 : kD / 32, kLanes = 32 / G;
+  const int lane = threadIdx.x & 31;
+  __syncwarp();  // the codes stored before come first
+  for (int n0 = warp * kRowsPerWarp * G; n0 < (warp + 1) * kRowsPerWarp * G; n0 += 32) {
+    const int n_here = min(32, kRowsPerWarp * G);
+    uint32_t odd = __ballot_sync(0xffffffffu, lane < n_here && !(s_row[n0 + min(lane, n_here - 1)].y > 0.f));
+    while (odd) {  // G groups at a time
+      uint32_t mine = odd;
+#pragma unroll
+      for (int i = 0; i < G; ++i) {
+        if (i < lane / kLanes) mine &= mine - 1;
+        odd &= odd - 1;
+      }
+      if (mine == 0) continue;
+      const int n = n0 + __ffs(mine) - 1, row = n / G, ch = (n & (G - 1)) * (kD / G) + 4 * (lane & (kLanes - 1));
+      const float4 g = s_row[n];
+      uint32_t w = 0;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) w |= code_exact(value_of<DT>(tile + row * (kD * 2) + 2 * (ch + e)), g.x, -g.w, levels) << (BITS * e);
+      uint8_t* const o = codes + (row * kD + ch) * BITS / 8;
+      if (BITS == 8) *reinterpret_cast<uint32_t*>(o) = w;
+      else *reinterpret_cast<uint16_t*>(o) = (uint16_t)w;
+    }
+  }
+}
 
 template <int DT, typename Jobs>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -412,6 +475,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       __syncwarp();
       // ---- (scale, min) and reciprocal of the warp's rows, a (row, group) per lane
+      bool odd = false;
 #pragma unroll
       for (int n0 = 0; n0 < kRowsPerWarp * G; n0 += 32) {
         const int n = n0 + lane;
@@ -426,8 +490,10 @@ __global__ void __launch_bounds__(kThreads, 1)
           store_meta(td.meta, rg, s, mn, meta16);
           const float y = reciprocal(s);
           s_row[rg] = make_float4(mn, y, y * fmaf(-y, s, 1.f), -s);
+          odd |= !(y > 0.f);
         }
       }
+      odd = __any_sync(0xffffffffu, odd);
       __syncwarp();
       // ---- codes
       uint8_t* const out_r = td.codes + r0 * (kD * BITS / 8) + lj * BITS;
@@ -447,22 +513,13 @@ __global__ void __launch_bounds__(kThreads, 1)
             code_pair(unpack2<DT>(w[p][2 * i + 1]), mn2, y2, yl2, ns2, mq[2], mq[3]);
             cw[i] = BITS == 8 ? pack4_u8(mq) : pack4_u4(mq);
           }
-          if (!(g.y > 0.f)) {  // outside the reciprocal's range
-#pragma unroll 1
-            for (int i = 0; i < 2; ++i) {
-              uint32_t c = 0;
-#pragma unroll 1
-              for (int e = 0; e < 4; ++e)
-                c |= code_exact(value_of<DT>(tile_r + it * 4 * (kD * 2) + 128 * p + 8 * i + 2 * e), g.x, -g.w, levels) << (BITS * e);
-              if (i == 0) cw[0] = c; else cw[1] = c;
-            }
-          }
           if (BITS == 8)
             *reinterpret_cast<uint2*>(out_r + it * 4 * kD + 64 * p) = make_uint2(cw[0], cw[1]);
           else
             *reinterpret_cast<uint32_t*>(out_r + it * 4 * (kD / 2) + 32 * p) = cw[0] | (cw[1] << 16);
         }
       }
+      if (odd) redo_values<DT, BITS>(tile, s_row, td.codes, warp);
     };
 
     auto keys = [&](auto bits_tag, auto rot_tag) {
@@ -577,48 +634,28 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int q = 0; q < 2; ++q) yl2[side][q] = f2_mul(y2[side][q], f2_fma(y2[side][q], ns2[side][q], one2));
         y_min = min3(y_min, fminf(b.x, b.y), fminf(b.z, b.w));
       }
-      if (y_min > 0.f) {
-#pragma unroll 2
-        for (int i = 0; i < kTok; ++i, o += 2 * row_stride) {
-          uint64_t v[2][2];
-          if (ROT) {
-            float x[8];
-            rotated(i, x);
-            v[0][0] = f2_pack(x[0], x[1]), v[0][1] = f2_pack(x[2], x[3]), v[1][0] = f2_pack(x[4], x[5]), v[1][1] = f2_pack(x[6], x[7]);
-          } else {
-            const uint2 wl = words(i, 0), wh = words(i, 1);
-            v[0][0] = unpack2<DT>(wl.x), v[0][1] = unpack2<DT>(wl.y), v[1][0] = unpack2<DT>(wh.x), v[1][1] = unpack2<DT>(wh.y);
-          }
-#pragma unroll
-          for (int side = 0; side < 2; ++side) {
-            uint32_t mq[4];
-            code_pair(v[side][0], mn2[side][0], y2[side][0], yl2[side][0], ns2[side][0], mq[0], mq[1]);
-            code_pair(v[side][1], mn2[side][1], y2[side][1], yl2[side][1], ns2[side][1], mq[2], mq[3]);
-            if (BITS == 8) *reinterpret_cast<uint32_t*>(o + side * (kD / 2)) = pack4_u8(mq);
-            else *reinterpret_cast<uint16_t*>(o + side * (kD / 4)) = (uint16_t)pack4_u4(mq);
-          }
+      const bool odd = __any_sync(0xffffffffu, !(y_min > 0.f));
+#pragma unroll 4
+      for (int i = 0; i < kTok; ++i, o += 2 * row_stride) {
+        uint64_t v[2][2];
+        if (ROT) {
+          float x[8];
+          rotated(i, x);
+          v[0][0] = f2_pack(x[0], x[1]), v[0][1] = f2_pack(x[2], x[3]), v[1][0] = f2_pack(x[4], x[5]), v[1][1] = f2_pack(x[6], x[7]);
+        } else {
+          const uint2 wl = words(i, 0), wh = words(i, 1);
+          v[0][0] = unpack2<DT>(wl.x), v[0][1] = unpack2<DT>(wl.y), v[1][0] = unpack2<DT>(wh.x), v[1][1] = unpack2<DT>(wh.y);
         }
-      } else {  // a group outside the reciprocal's range
-#pragma unroll 1
-        for (int n = 0; n < 2 * kTok; ++n) {  // token and side
-          const int side = n & 1;
-          uint32_t w = 0;
-#pragma unroll 1
-          for (int e = 0; e < 4; ++e) {
-            const uint8_t* const at_ch = row0 + (n >> 1) * (2 * kD * 2) + 2 * e;  // the low channel; its partner 64 channels on
-            float v = value_of<DT>(at_ch + side * kD);
-            if (ROT) {  // the operations above
-              const float2 r = s_rot[td.rot][4 * p + e];
-              v = fmaf(v, r.x, __fmul_rn(value_of<DT>(at_ch + (side ^ 1) * kD), side ? -r.y : r.y));
-            }
-            const int gc = gp + side * (kD / 2) + e;
-            w |= code_exact(v, s_par[0][gc], -s_par[2][gc], levels) << (BITS * e);
-          }
-          uint8_t* const at_o = o + (n >> 1) * 2 * row_stride + side * (kD / 2 * BITS / 8);
-          if (BITS == 8) *reinterpret_cast<uint32_t*>(at_o) = w;
-          else *reinterpret_cast<uint16_t*>(at_o) = (uint16_t)w;
+#pragma unroll
+        for (int side = 0; side < 2; ++side) {
+          uint32_t mq[4];
+          code_pair(v[side][0], mn2[side][0], y2[side][0], yl2[side][0], ns2[side][0], mq[0], mq[1]);
+          code_pair(v[side][1], mn2[side][1], y2[side][1], yl2[side][1], ns2[side][1], mq[2], mq[3]);
+          if (BITS == 8) *reinterpret_cast<uint32_t*>(o + side * (kD / 2)) = pack4_u8(mq);
+          else *reinterpret_cast<uint16_t*>(o + side * (kD / 4)) = (uint16_t)pack4_u4(mq);
         }
       }
+      if (odd) redo_keys<DT, BITS, ROT>(tile, s_par, s_rot[ROT ? td.rot : 0], td.codes, row_stride, warp);
     };
 
     using std::integral_constant;

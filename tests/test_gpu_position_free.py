@@ -273,3 +273,46 @@ def test_quantiser_whose_loads_stop_reports_it_and_writes_nothing_else(Hkv, bits
             assert torch.equal(got, whole)
     finally:
         B.kvb_destroy(ctx)
+
+
+@pytest.mark.parametrize("Hkv", [1, 2])
+@pytest.mark.parametrize("bits", [8, 4])
+@pytest.mark.parametrize("pos", [-1, 4096 + 128])
+@pytest.mark.parametrize("lattice", [False, True])
+def test_scales_of_every_magnitude(Hkv, bits, pos, lattice):
+    """Channels and rows whose scales spread over all that bfloat16 holds, on both sides of the range in which the
+    reciprocal decides, alone among ordinary ones and all over; a lattice whose every other quotient is a tie.  Codes and
+    metadata equal the oracle's bit for bit, rotated keys too (a channel's partner has another magnitude)."""
+    sh = synth.Shape(L=2, Hq=Hkv, Hkv=Hkv)
+    top = 2 * ((1 << bits) - 1)
+    g = torch.Generator().manual_seed(bits + 100 * Hkv)
+    ctx = B.create_for_shape(sh, 0)
+    try:
+        if lattice:
+            k, v = (torch.randint(0, top // 2 + 1, (sh.L, sh.C, Hkv, sh.d), generator=g).float() for _ in range(2))
+            k[:, 0::32], k[:, 1::32] = 0.0, float(top)
+            v[..., 0::32], v[..., 1::32] = 0.0, float(top)
+        else:
+            k, v = (torch.randn((sh.L, sh.C, Hkv, sh.d), generator=g) for _ in range(2))
+        e = torch.linspace(-120, 116, 128).round()
+        edges = torch.tensor([-106, -105, -104, -103, -102, -101, -100, -99, -98, 90, 91, 92, 93, 94, 95, 96, 97, 98, 99, 100])
+        e[10 : 10 + len(edges)] = edges.float()  # scales about 1e-30 and 1e30 for ranges of 16 and 256 steps
+        e = e[torch.randperm(128, generator=g)]
+        k[0] *= torch.exp2(e)             # layer 0: every channel and every row another magnitude
+        v[0] *= torch.exp2(e).view(-1, 1, 1)
+        k[1, ..., 70] *= 2.0**-110        # layer 1: one of either among ordinary ones
+        v[1, 70] *= 2.0**110
+        k, v = k.to(sh.torch_dtype), v.to(sh.torch_dtype)
+        G = 1 if bits == 8 else 4
+        out = dict(k_codes=torch.zeros((sh.L, sh.C, Hkv, sh.d * bits // 8), dtype=torch.uint8, device=DEV), k_meta=torch.zeros((sh.L, G, Hkv, sh.d, 2), device=DEV),
+                   v_codes=torch.zeros((sh.L, sh.C, Hkv, sh.d * bits // 8), dtype=torch.uint8, device=DEV), v_meta=torch.zeros((sh.L, sh.C, Hkv, G, 2), device=DEV))
+        B.kvb_quantize_chunks(ctx, [dict(bits=bits, k=k.to(DEV), v=v.to(DEV), unrotate_from=pos, **out)])
+        B.kvb_last_status(ctx)
+        gk, gv = (sh.C, sh.d) if bits == 8 else (sh.int4_group, sh.int4_group)
+        for l in range(sh.L):
+            u = oracle.unrotate_keys(helpers.bits_of(k)[l], helpers.dt_code(sh), sh.theta, pos) if pos >= 0 else helpers.f64_of(k)[l]
+            for side, (codes, meta) in (("k", oracle.quantize_k(u, bits, gk)), ("v", oracle.quantize_v(helpers.f64_of(v)[l], bits, gv))):
+                assert np.array_equal(out[side + "_codes"][l].cpu().numpy(), codes), (side, l)
+                assert np.array_equal(out[side + "_meta"][l].cpu().numpy(), meta), (side, l)
+    finally:
+        B.kvb_destroy(ctx)

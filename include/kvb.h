@@ -210,7 +210,9 @@ int kvb_chunk_importance(kvb_ctx* ctx, const kvb_request* reqs, int n_req, float
 
 /* KV Quantization, Eq. 6 (cache-population side), for one chunk: x [L][C][H][d]
  * in kv_dtype (device) -> codes and (scale, min) metadata in the layouts above.
- * is_value = 0: keys, per channel; 1: values, per token.  bits: 4 or 8. */
+ * is_value = 0: keys, per channel; 1: values, per token.  bits: 4 or 8.
+ * A NaN is left out of its group's extremes and has code 0, as has every finite
+ * value of a group with an infinite scale. */
 int kvb_quantize_chunk(kvb_ctx* ctx, const void* x, int is_value, int bits, void* codes, void* meta,
                        void* cuda_stream);
 

@@ -142,16 +142,28 @@ __device__ __noinline__ uint32_t code_exact(float v, float mn, float s, float le
 }
 // y = RN(1 / s); the rest of the reciprocal is y (1 - y s).  Within 1e-30 .. 1e30 code_pair's remainder is exact for every
 // quotient that can decide (from 1/4 on it is a multiple of 2^-25 2^-23 2^-100, above float32's smallest number) and nothing
-// overflows.  Outside, or where the extremes are not finite, y is zero, and the IEEE division decides for the group.
+// overflows.  Outside, and in a group with a value that is no number or whose minimum is infinite, y is zero, and the IEEE
+// division decides for the group: a NaN gets code 0, and so do the values of a group without a finite one.
 __device__ __forceinline__ float reciprocal(float s) { return s >= 1e-30f && s <= 1e30f ? __frcp_rn(s) : 0.f; }
-__device__ __forceinline__ float min3(float a, float b, float c) {
+// minimum / maximum of two or three values in which a NaN stays
+__device__ __forceinline__ float min_nan(float a, float b) {
   float d;
-  asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
   return d;
 }
-__device__ __forceinline__ float max3(float a, float b, float c) {
+__device__ __forceinline__ float max_nan(float a, float b) {
   float d;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+  return d;
+}
+__device__ __forceinline__ float min_nan(float a, float b, float c) {
+  float d;
+  asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+__device__ __forceinline__ float max_nan(float a, float b, float c) {
+  float d;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
 // four codes, each in the low byte of m_i, as one word (code 0 in the lowest byte)
@@ -170,15 +182,15 @@ __device__ __forceinline__ uint64_t unpack2(uint32_t w) {
   const float2 t = __half22float2(*reinterpret_cast<const __half2*>(&w));
   return f2_pack(t.x, t.y);
 }
-// element-wise minimum / maximum of two words of two 16-bit values each (exact: no rounding is involved)
+// element-wise minimum / maximum of two words of two 16-bit values each (exact: no rounding is involved; a NaN stays)
 template <int DT>
 __device__ __forceinline__ uint32_t min2_16(uint32_t a, uint32_t b) {
   uint32_t r;
   if (DT == KVB_DT_BF16) {
-    const __nv_bfloat162 t = __hmin2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
+    const __nv_bfloat162 t = __hmin2_nan(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
     r = *reinterpret_cast<const uint32_t*>(&t);
   } else {
-    const __half2 t = __hmin2(*reinterpret_cast<const __half2*>(&a), *reinterpret_cast<const __half2*>(&b));
+    const __half2 t = __hmin2_nan(*reinterpret_cast<const __half2*>(&a), *reinterpret_cast<const __half2*>(&b));
     r = *reinterpret_cast<const uint32_t*>(&t);
   }
   return r;
@@ -187,10 +199,10 @@ template <int DT>
 __device__ __forceinline__ uint32_t max2_16(uint32_t a, uint32_t b) {
   uint32_t r;
   if (DT == KVB_DT_BF16) {
-    const __nv_bfloat162 t = __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
+    const __nv_bfloat162 t = __hmax2_nan(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
     r = *reinterpret_cast<const uint32_t*>(&t);
   } else {
-    const __half2 t = __hmax2(*reinterpret_cast<const __half2*>(&a), *reinterpret_cast<const __half2*>(&b));
+    const __half2 t = __hmax2_nan(*reinterpret_cast<const __half2*>(&a), *reinterpret_cast<const __half2*>(&b));
     r = *reinterpret_cast<const uint32_t*>(&t);
   }
   return r;
@@ -201,6 +213,22 @@ __device__ __forceinline__ float value_of(const void* p) {
   float a, b;
   f2_unpack(unpack2<DT>(*reinterpret_cast<const uint16_t*>(p)), a, b);
   return a;
+}
+
+// The extremes of a group with a NaN among its N values (16 bits each, STRIDE bytes apart): those of the others.  Rotated
+// keys: r is the channel's cos / sin, the partner's value lies `partner` bytes on.  A group of NaNs alone has the minimum NaN,
+// rotated keys +inf.
+template <int DT, bool ROT, int N, int STRIDE>
+__device__ __noinline__ float2 number_extremes(const uint8_t* x, const float2* r, int partner) {
+  const uint16_t none = 0x7FFF;
+  float mn = ROT ? INFINITY : value_of<DT>(&none), mx = ROT ? -INFINITY : mn;
+#pragma unroll 16
+  for (int i = 0; i < N; ++i, x += STRIDE) {
+    float v = value_of<DT>(x);
+    if (ROT) v = fmaf(v, r->x, __fmul_rn(value_of<DT>(x + partner), partner < 0 ? -r->y : r->y));  // as in the kernel
+    mn = fminf(mn, v), mx = fmaxf(mx, v);
+  }
+  return make_float2(mn, mx);
 }
 
 // (scale, min) of a group from its extremes.  Compact metadata: min is rounded down to binary16
@@ -485,10 +513,15 @@ __global__ void __launch_bounds__(kThreads, 1)
           float a, b, c, d, s;
           f2_unpack(unpack2<DT>(ext.x), a, b);
           f2_unpack(unpack2<DT>(ext.y), c, d);
-          float mn = fminf(a, b);
-          group_params(mn, fmaxf(c, d), levels, meta16, s);
+          float mn = min_nan(a, b), mx = max_nan(c, d);
+          const bool numbers = fabsf(mn) < INFINITY;
+          if (mn != mn) {
+            const float2 e = number_extremes<DT, false, kD / G, 2>(tile + rg * (kD / G * 2), nullptr, 0);
+            mn = e.x, mx = e.y;
+          }
+          group_params(mn, mx, levels, meta16, s);
           store_meta(td.meta, rg, s, mn, meta16);
-          const float y = reciprocal(s);
+          const float y = numbers ? reciprocal(s) : 0.f;
           s_row[rg] = make_float4(mn, y, y * fmaf(-y, s, 1.f), -s);
           odd |= !(y > 0.f);
         }
@@ -564,14 +597,14 @@ __global__ void __launch_bounds__(kThreads, 1)
           rotated(i + 1, v[1]);
 #pragma unroll
           for (int c = 0; c < 8; ++c) {
-            mn[c] = i == 0 ? fminf(v[0][c], v[1][c]) : min3(mn[c], v[0][c], v[1][c]);
-            mx[c] = i == 0 ? fmaxf(v[0][c], v[1][c]) : max3(mx[c], v[0][c], v[1][c]);
+            mn[c] = i == 0 ? min_nan(v[0][c], v[1][c]) : min_nan(mn[c], v[0][c], v[1][c]);
+            mx[c] = i == 0 ? max_nan(v[0][c], v[1][c]) : max_nan(mx[c], v[0][c], v[1][c]);
           }
         }
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
           const float other = __shfl_xor_sync(0xffffffffu, half ? mn[c] : mx[c], 16);
-          mn[c] = half ? fmaxf(mx[c], other) : fminf(mn[c], other);
+          mn[c] = half ? max_nan(mx[c], other) : min_nan(mn[c], other);
         }
         ext[0] = make_float4(mn[0], mn[1], mn[2], mn[3]), ext[1] = make_float4(mn[4], mn[5], mn[6], mn[7]);
       } else {
@@ -606,13 +639,18 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int i = 0; i < kWarps / (G == 1 ? 2 : G); ++i) {
           const int w = G == 1 ? sub + 2 * i : kWarps / G * sub + i;
           const float lo = s_ext[ext_at(w, 0, ch)], hi = s_ext[ext_at(w, 1, ch)];
-          a = i == 0 ? lo : fminf(a, lo), b = i == 0 ? hi : fmaxf(b, hi);
+          a = i == 0 ? lo : min_nan(a, lo), b = i == 0 ? hi : max_nan(b, hi);
         }
-        if (G == 1) a = fminf(a, __shfl_xor_sync(0xffffffffu, a, 1)), b = fmaxf(b, __shfl_xor_sync(0xffffffffu, b, 1));
-        group_params(a, b, levels, meta16, s);
+        if (G == 1) a = min_nan(a, __shfl_xor_sync(0xffffffffu, a, 1)), b = max_nan(b, __shfl_xor_sync(0xffffffffu, b, 1));
         const int g = G == 1 ? 0 : sub;
+        const bool numbers = fabsf(a) < INFINITY;
+        if (a != a) {
+          const float2 e = number_extremes<DT, ROT, kGroupTokens, kD * 2>(tile + g * kGroupTokens * (kD * 2) + 2 * ch, &s_rot[ROT ? td.rot : 0][ch & (kD / 2 - 1)], ch < kD / 2 ? kD : -kD);
+          a = e.x, b = e.y;
+        }
+        group_params(a, b, levels, meta16, s);
         if (G > 1 || sub == 0) {
-          s_par[0][g * kD + ch] = a, s_par[1][g * kD + ch] = reciprocal(s), s_par[2][g * kD + ch] = -s;
+          s_par[0][g * kD + ch] = a, s_par[1][g * kD + ch] = numbers ? reciprocal(s) : 0.f, s_par[2][g * kD + ch] = -s;
           store_meta(td.meta, (uint32_t)(g * H * kD + ch), s, a, meta16);
         }
       }
@@ -632,7 +670,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         ns2[side][0] = f2_pack(c.x, c.y), ns2[side][1] = f2_pack(c.z, c.w);
 #pragma unroll
         for (int q = 0; q < 2; ++q) yl2[side][q] = f2_mul(y2[side][q], f2_fma(y2[side][q], ns2[side][q], one2));
-        y_min = min3(y_min, fminf(b.x, b.y), fminf(b.z, b.w));
+        y_min = fminf(y_min, fminf(fminf(b.x, b.y), fminf(b.z, b.w)));
       }
       const bool odd = __any_sync(0xffffffffu, !(y_min > 0.f));
 #pragma unroll 4

@@ -316,3 +316,61 @@ def test_scales_of_every_magnitude(Hkv, bits, pos, lattice):
                 assert np.array_equal(out[side + "_meta"][l].cpu().numpy(), meta), (side, l)
     finally:
         B.kvb_destroy(ctx)
+
+
+def _eq6_of_numbers(x, bits):
+    """Eq. 6 on [..., group] rows with the NaNs left out of the extremes; a quotient that is no number gives code 0."""
+    x = x.float()
+    nan = torch.isnan(x)
+    mn = torch.where(nan, float("inf"), x).amin(-1, keepdim=True)
+    mx = torch.where(nan, -float("inf"), x).amax(-1, keepdim=True)
+    s = torch.where(mx > mn, (mx - mn) / float(2**bits - 1), torch.ones_like(mn))
+    codes = torch.round((x - mn) / s)
+    return torch.where(torch.isnan(codes), 0.0, torch.clamp(codes, 0, 2**bits - 1)), s, mn
+
+
+@pytest.mark.parametrize("kv_dtype", ["bf16", "fp16"])
+@pytest.mark.parametrize("bits", [8, 4])
+@pytest.mark.parametrize("rotated", [False, True])
+def test_values_that_are_no_numbers_stay_in_their_place(kv_dtype, bits, rotated):
+    """NaN and infinity in even and odd channels, alone and all over a group, keys and values: codes and metadata equal
+    Eq. 6 bit for bit, those of the groups beside it among them, and a NaN has code 0."""
+    sh = synth.Shape(L=1, Hq=2, Hkv=2, kv_dtype=kv_dtype)
+    nan, inf = float("nan"), float("inf")
+    ctx = B.create_for_shape(sh, 0)
+    try:
+        g = torch.Generator().manual_seed(17)
+        k, v = (torch.randn((sh.L, sh.C, sh.Hkv, sh.d), generator=g) for _ in range(2))
+        for i, c in enumerate((4, 9, 14, 19)):  # every parity and place of a thread's four channels
+            k[:, 5 + 31 * i, :, c] = nan
+            v[:, 3 + i, :, c + 32 * (i & 1)] = nan
+        k[:, 70, :, 24], k[:, 71, :, 27], k[:, 72, :, 33], k[:, 73, :, 33] = inf, -inf, inf, -inf
+        k[..., 40], k[..., 41], k[..., 50] = inf, -inf, nan
+        v[:, 10, :, 10], v[:, 11, :, 11], v[:, 12, :, 64], v[:, 12, :, 67] = inf, -inf, inf, -inf
+        v[:, 13], v[:, 14], v[:, 15] = inf, -inf, nan
+        k, v = k.to(sh.torch_dtype), v.to(sh.torch_dtype)
+        G = 1 if bits == 8 else 4
+        out = dict(k_codes=torch.zeros((sh.L, sh.C, sh.Hkv, sh.d * bits // 8), dtype=torch.uint8, device=DEV), k_meta=torch.zeros((sh.L, G, sh.Hkv, sh.d, 2), device=DEV),
+                   v_codes=torch.zeros((sh.L, sh.C, sh.Hkv, sh.d * bits // 8), dtype=torch.uint8, device=DEV), v_meta=torch.zeros((sh.L, sh.C, sh.Hkv, G, 2), device=DEV))
+        B.kvb_quantize_chunks(ctx, [dict(bits=bits, k=k.to(DEV), v=v.to(DEV), unrotate_from=0 if rotated else -1, **out)])
+        B.kvb_last_status(ctx)
+        u = k.float()
+        if rotated:  # by the angle 0: cos 1, sin 0 (0 times infinity is no number)
+            lo, hi = u[..., :64], u[..., 64:]
+            u = torch.cat([lo + hi * 0.0, hi + lo * -0.0], -1)
+        x = {"k": u.view(sh.L, G, sh.C // G, sh.Hkv, sh.d).permute(0, 1, 3, 4, 2), "v": v.float().view(sh.L, sh.C, sh.Hkv, G, sh.d // G)}
+        back = {"k": lambda t: t.permute(0, 1, 4, 2, 3).reshape(k.shape), "v": lambda t: t.reshape(v.shape)}
+        for side in ("k", "v"):
+            codes, s, mn = _eq6_of_numbers(x[side], bits)
+            none = torch.isnan(x[side]).all(-1, keepdim=True)  # a group without a number
+            if side == "v" or not rotated:
+                mn = torch.where(none, nan, mn)
+            else:
+                assert torch.equal(mn[none], torch.full_like(mn[none], inf))
+            got = out[side + "_codes"].cpu()
+            if bits == 4:
+                got = torch.stack([got & 15, got >> 4], -1).flatten(-2)
+            assert bool((torch.isnan(x[side]) & ~none).any()) and torch.equal(got, back[side](codes).to(torch.uint8))
+            np.testing.assert_array_equal(out[side + "_meta"].cpu().numpy(), torch.stack([s[..., 0], mn[..., 0]], -1).numpy())
+    finally:
+        B.kvb_destroy(ctx)

@@ -49,6 +49,11 @@ constexpr uint32_t kTileBytes = kRows * kD * 2;
 constexpr uint32_t kWaitLimit = 1u << 22;         // polls after which a wait gives up
 constexpr uint32_t kStalledWaitLimit = 1u << 10;  // the same in a launch whose fetching warps are made to stop (option quantize_stalled_fetch)
 constexpr int kStages = 5;     // tile buffers: one in work per group, the others in flight
+// Barriers on which tiles land, two for each group: tile t of a CTA has barrier t mod 6, lap t / 6.  (One per buffer would not
+// do.  A wait goes by the parity of the lap, so whoever waits for a lap must know that the one before is over.  The barrier's
+// tile before, t - 6, is the same group's: the warp has worked on it.  The buffer's tile before, t - 5, is another group's, and
+// copies land in any order: a warp that is early would take its parity for its own tile's.)
+constexpr int kLandings = 2 * kGroups;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
@@ -366,7 +371,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ __align__(16) float s_par_all[kGroups][3][4 * kD];        // keys: min, reciprocal and -scale of every [token group][channel]
   __shared__ float2 s_rot[kStages][kD / 2];               // cos / sin of a chunk's rotation; a ring, in use by at most kStages tiles
   __shared__ TileDesc s_tile[kStages];
-  __shared__ __align__(8) uint64_t s_full[kStages], s_empty[kStages];
+  __shared__ __align__(8) uint64_t s_full[kLandings], s_empty[kStages];
   __shared__ uint32_t s_gave_up[kGroups];  // warps of the group whose wait for the tile ran out
   const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) & (kWarps - 1), group = threadIdx.x / (kWarps * 32);
   const int tid = threadIdx.x & (kWarps * 32 - 1);  // within the group
@@ -376,9 +381,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t first = (uint32_t)((unsigned long long)n_items * blockIdx.x / gridDim.x);
   const uint32_t last = (uint32_t)((unsigned long long)n_items * (blockIdx.x + 1) / gridDim.x);
 
-  if (threadIdx.x < kStages) {
+  if (threadIdx.x < kLandings) {
     mbar_init(&s_full[threadIdx.x], kFetchers);
-    mbar_init(&s_empty[threadIdx.x], kWarps);
+    if (threadIdx.x < kStages) mbar_init(&s_empty[threadIdx.x], kWarps);
     if (threadIdx.x < kGroups) s_gave_up[threadIdx.x] = 0;
   }
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -393,6 +398,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // ------------------------------ the fetching warps: descriptors, rotation tables and copies, up to kStages tiles ahead
     Tile t(first, log_h, m.L);
     uint32_t rot_job = 0xFFFFFFFFu, stage = 0, phase = 1;  // a fresh barrier passes a wait for the phase before its first
+    uint32_t landing = 0, lap = 0;                         // the tile's barrier and the parity of its lap
     int rot_buf = 0;
     uint32_t left = stalled ? blockIdx.x % (2 * kStages) : 0xFFFFFFFFu;  // tiles until a stalled fetch
     for (uint32_t item = first; item < last + kGroups; ++item, t.next(H, m.L)) {
@@ -415,7 +421,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!mbar_wait(&s_empty[stage], phase, limit)) {
         if (lane == 0) atomicOr(status, DEV_STATUS_WAIT_TIMEOUT);
         asm volatile("cp.async.wait_all;" ::: "memory");  // the copies in flight land before their buffers are given up
-        for (uint32_t i = 0; i < kStages; ++i) mbar_wait(&s_full[i], i < stage ? phase ^ 1u : phase, limit);
+        for (uint32_t i = 0; i < kLandings; ++i) mbar_wait(&s_full[i], i < landing ? lap : lap ^ 1u, limit);
         return;
       }
       if (!end && !t.kv && job_at(jobs, t.job).unrotate_from >= 0) {
@@ -437,18 +443,19 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint8_t* g = x + (size_t)(tid >> 4) * H * (kD * 2) + (tid & 15) * 16;
 #pragma unroll 4
         for (int i = 0; i < (int)kTileBytes / 16; i += kFetchers * 32, g += (size_t)(kFetchers * 2) * H * (kD * 2)) cp_async16(dst + (i + tid) * 16, g);
-        cp_async_arrive(&s_full[stage]);
+        cp_async_arrive(&s_full[landing]);
       }
       __syncwarp();
       if (lane == 0) {
-        if (end || !bulk || tid != 0) mbar_arrive(&s_full[stage]);
+        if (end || !bulk || tid != 0) mbar_arrive(&s_full[landing]);
         else {  // one contiguous block
-          mbar_expect_tx(&s_full[stage], kTileBytes);
+          mbar_expect_tx(&s_full[landing], kTileBytes);
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the buffer's previous tile may have come by cp.async
-          bulk_g2s(dst, x, kTileBytes, &s_full[stage]);
+          bulk_g2s(dst, x, kTileBytes, &s_full[landing]);
         }
       }
       if (++stage == kStages) stage = 0, phase ^= 1;
+      if (++landing == kLandings) landing = 0, lap ^= 1;
     }
     return;
   }
@@ -456,11 +463,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   // ------------------------------ the others.  Between two tiles they meet only where data changes hands: inside a keys tile.
   float* const s_ext = s_ext_all[group];
   float (*const s_par)[4 * kD] = s_par_all[group];
-  uint32_t phase = 0;
+  uint32_t mine = 0;  // tiles of the group so far, mod 4
   for (uint32_t stage = group;;) {  // every kGroups-th tile
-    if (!mbar_wait(&s_full[stage], phase, limit)) {
+    if (!mbar_wait(&s_full[group + kGroups * (mine & 1)], mine >> 1, limit)) {
       if (lane == 0) atomicOr(status, DEV_STATUS_WAIT_TIMEOUT);
-      if (!landed_late(&s_full[stage], phase, limit, &s_gave_up[group])) return;
+      if (!landed_late(&s_full[group + kGroups * (mine & 1)], mine >> 1, limit, &s_gave_up[group])) return;
     }
     const TileDesc td = s_tile[stage];
     if (!td.codes) break;
@@ -710,7 +717,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncwarp();
     if (lane == 0) mbar_arrive(&s_empty[stage]);
     stage += kGroups;
-    if (stage >= kStages) stage -= kStages, phase ^= 1;
+    if (stage >= kStages) stage -= kStages;
+    mine = (mine + 1) & 3;
   }
 }
 

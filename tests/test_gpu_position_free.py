@@ -374,3 +374,38 @@ def test_values_that_are_no_numbers_stay_in_their_place(kv_dtype, bits, rotated)
             np.testing.assert_array_equal(out[side + "_meta"].cpu().numpy(), torch.stack([s[..., 0], mn[..., 0]], -1).numpy())
     finally:
         B.kvb_destroy(ctx)
+
+
+@pytest.mark.parametrize("side", ["k", "v"])
+@pytest.mark.parametrize("Hkv", [1, 16])
+def test_long_runs_of_one_side(side, Hkv):
+    """Sixteen chunks of 36 layers, one side only, again and again: tens of tiles for every CTA, all of a kind, as fast as
+    they come, so that loads land out of order and the warps of a group drift apart.  Codes and metadata of every call equal
+    Eq. 6 bit for bit."""
+    sh = synth.Shape(L=36, Hq=16, Hkv=Hkv)
+    n = 256 // Hkv
+    ctx = B.create_for_shape(sh, 0)
+    try:
+        g = torch.Generator(device=DEV).manual_seed(5)
+        x = torch.empty((n, sh.L, sh.C, Hkv, sh.d), dtype=sh.torch_dtype, device=DEV)
+        want_codes = torch.empty(x.shape, dtype=torch.uint8, device=DEV)
+        meta_shape = (n, sh.L, 1, Hkv, sh.d, 2) if side == "k" else (n, sh.L, sh.C, Hkv, 1, 2)
+        want_meta = torch.empty(meta_shape, device=DEV)
+        for i in range(n):
+            x[i] = torch.randn(x.shape[1:], generator=g, device=DEV)
+            rows = x[i].permute(0, 2, 3, 1) if side == "k" else x[i]  # tokens, or channels, last
+            mn, mx = rows.float().amin(-1, keepdim=True), rows.float().amax(-1, keepdim=True)
+            s = (mx - mn) / torch.full_like(mn, 255.0)  # (a division by a number would be a multiplication by its reciprocal)
+            codes = torch.round((rows.float() - mn) / s)
+            want_codes[i] = codes.permute(0, 3, 1, 2) if side == "k" else codes
+            want_meta[i] = torch.cat([s, mn], -1).view(meta_shape[1:])
+        codes, meta = torch.empty_like(want_codes), torch.empty_like(want_meta)
+        jobs = B.QuantizeTable([{"bits": 8, side: x[i], side + "_codes": codes[i], side + "_meta": meta[i]} for i in range(n)])
+        for _ in range(20):
+            codes.zero_(), meta.zero_()
+            for _ in range(5):
+                B.kvb_quantize_chunks(ctx, jobs)
+            B.kvb_last_status(ctx)
+            assert torch.equal(codes, want_codes) and torch.equal(meta, want_meta)
+    finally:
+        B.kvb_destroy(ctx)

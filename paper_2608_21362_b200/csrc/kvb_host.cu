@@ -742,17 +742,26 @@ int kvb_quantize_chunks(kvb_ctx* c, const kvb_quantize_job* jobs, int n_jobs, vo
   }
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   KVB_CUDA(c, cudaSetDevice(c->device));
+  // the wanted tiles: one per layer, KV head and side
+  const auto tiles_of = [&](const kvb_quantize_job& j) { return (long long)c->dims.L * c->dims.Hkv * ((j.k != nullptr) + (j.v != nullptr)); };
+  long long n_tiles = 0;
+  bool equal = true;
+  for (int i = 0; i < n_jobs; ++i) n_tiles += tiles_of(jobs[i]), equal = equal && tiles_of(jobs[i]) == tiles_of(jobs[0]);
+  if (n_tiles > 0xFFFFFFF0ll) return fail(c, KVB_ERR_CUDA, "%lld tiles in one call", n_tiles);
+  const QuantBatch batch{(uint32_t)n_jobs, (uint32_t)n_tiles, equal ? (uint32_t)tiles_of(jobs[0]) : 0u};
   auto fill = [&](QuantJob* qj) {
+    uint32_t at = 0;
     for (int i = 0; i < n_jobs; ++i) {
       const kvb_quantize_job& j = jobs[i];
-      qj[i] = QuantJob{j.k, j.v, j.k_codes, j.v_codes, j.k_meta, j.v_meta, j.bits, j.unrotate_from, j.meta_fp16, 0};
+      qj[i] = QuantJob{j.k, j.v, j.k_codes, j.v_codes, j.k_meta, j.v_meta, j.bits, j.unrotate_from, j.meta_fp16, at};
+      at += (uint32_t)tiles_of(j);
     }
   };
   if (n_jobs <= kQuantInline && !c->force_copy) {  // the jobs travel as the kernel's argument
     QuantJob qj[kQuantInline];
     fill(qj);
     c->last_stream = st;
-    KVB_CUDA(c, launch_quantize_inline(qj, n_jobs, c->dims, c->inv_freq, c->status_dev, c->n_sm, c->pdl, c->quant_stalled, st));
+    KVB_CUDA(c, launch_quantize_inline(qj, batch, c->dims, c->inv_freq, c->status_dev, c->n_sm, c->pdl, c->quant_stalled, st));
   } else {
     uint8_t* host = nullptr;
     const int slot_code = take_slot(c, &host);
@@ -762,7 +771,7 @@ int kvb_quantize_chunks(kvb_ctx* c, const kvb_quantize_job* jobs, int n_jobs, vo
     const int up = upload(c, slot, host, sizeof(QuantJob) * (size_t)n_jobs, st);
     if (up != KVB_OK) return up;
     c->last_stream = st;
-    KVB_CUDA(c, launch_quantize_table(reinterpret_cast<const QuantJob*>(c->arena_dev), n_jobs, c->dims, c->inv_freq, c->status_dev, c->n_sm, c->pdl, c->quant_stalled, st));
+    KVB_CUDA(c, launch_quantize_table(reinterpret_cast<const QuantJob*>(c->arena_dev), batch, c->dims, c->inv_freq, c->status_dev, c->n_sm, c->pdl, c->quant_stalled, st));
   }
   c->launches += 1;
   return KVB_OK;

@@ -154,15 +154,19 @@ struct QuantJob {
   int32_t bits;
   int32_t unrotate_from;  // >= 0 (keys only): rotate back by R^(-unrotate_from) before quantising
   int32_t meta16;
-  int32_t reserved;
+  uint32_t tile_offset;  // wanted tiles of the jobs before
+};
+// per_job: the tiles of every job, 0 where they differ
+struct QuantBatch {
+  uint32_t n_jobs, n_tiles, per_job;
 };
 // Up to kQuantInline jobs travel as the kernel's own argument (host_jobs is read before the call returns),
 // more through a table in device memory.  inv_freq: [d/2] doubles, device.  stalled: the fetching warps stop before they
 // are through and the waits are short (option quantize_stalled_fetch).
 constexpr int kQuantInline = (int)(kDescBlobBytes / sizeof(QuantJob));
-cudaError_t launch_quantize_inline(const QuantJob* host_jobs, int n_jobs, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl, bool stalled,
+cudaError_t launch_quantize_inline(const QuantJob* host_jobs, const QuantBatch& b, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl, bool stalled,
                                    cudaStream_t st);
-cudaError_t launch_quantize_table(const QuantJob* table, int n_jobs, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl, bool stalled,
+cudaError_t launch_quantize_table(const QuantJob* table, const QuantBatch& b, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl, bool stalled,
                                   cudaStream_t st);
 cudaError_t quantize_configure();
 

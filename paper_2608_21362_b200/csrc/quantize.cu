@@ -265,26 +265,49 @@ template <int N>
 __device__ __forceinline__ const QuantJob& job_at(const InlineJobs<N>& t, uint32_t j) { return t.d[j]; }
 __device__ __forceinline__ const QuantJob& job_at(const QuantJob* t, uint32_t j) { return t[j]; }
 
-// One tile of the batch; items are numbered job-major, then layer, then K|V, then the H tiles of a chunk-layer.
+// One tile of the batch.  The wanted tiles are numbered job-major, then layer, then K|V, then the H tiles of a chunk-layer; a
+// side that a job does not want has no numbers, so that the CTAs' ranges hold equal work.
 struct Tile {
   uint32_t job;
   int l, kv, h;
-  __device__ __forceinline__ Tile(uint32_t item, int log_h, int L) {
+  bool both;  // the job wants both sides
+  // per_job: the tiles of every job, 0 where they differ (then the job is the last one that starts at or before the item)
+  template <typename Jobs>
+  __device__ __forceinline__ Tile(const Jobs& jobs, uint32_t item, uint32_t n_jobs, uint32_t per_job, int log_h) {
+    if (per_job) {
+      job = item / per_job;
+    } else {
+      uint32_t lo = 0, hi = n_jobs - 1;
+      while (lo < hi) {
+        const uint32_t mid = (lo + hi + 1) >> 1;
+        if (job_at(jobs, mid).tile_offset <= item) lo = mid; else hi = mid - 1;
+      }
+      job = lo;
+    }
+    enter(jobs);
+    item -= job_at(jobs, job).tile_offset;
     h = (int)(item & ((1u << log_h) - 1u));
     item >>= log_h;
-    kv = (int)(item & 1u);
-    item >>= 1;
-    job = item / (uint32_t)L;
-    l = (int)(item - job * (uint32_t)L);
+    if (both) kv = (int)(item & 1u), item >>= 1;
+    l = (int)item;
   }
-  __device__ __forceinline__ void next(int H, int L) {
+  // to the first tile of `job`
+  template <typename Jobs>
+  __device__ __forceinline__ void enter(const Jobs& jobs) {
+    const QuantJob& jb = job_at(jobs, job);
+    l = 0, h = 0, kv = jb.k ? 0 : 1, both = jb.k && jb.v;
+  }
+  template <typename Jobs>
+  __device__ __forceinline__ void next(const Jobs& jobs, int H, int L, bool more) {
     if (++h < H) return;
     h = 0;
-    kv ^= 1;
-    if (kv) return;
-    if (++l < L) return;
-    l = 0;
+    if (both) {
+      kv ^= 1;
+      if (kv) return;
+    }
+    if (++l < L || !more) return;
     ++job;
+    enter(jobs);
   }
 };
 
@@ -364,7 +387,7 @@ __device__ __noinline__ void redo_values(const uint8_t* tile, const float4* s_ro
 
 template <int DT, typename Jobs>
 __global__ void __launch_bounds__(kThreads, 1)
-    quantize_batch_kernel(const __grid_constant__ Jobs jobs, ModelDims m, uint32_t n_items, const double* __restrict__ inv_freq,
+    quantize_batch_kernel(const __grid_constant__ Jobs jobs, ModelDims m, uint32_t n_jobs, uint32_t n_items, uint32_t per_job, const double* __restrict__ inv_freq,
                           uint32_t* __restrict__ status, bool stalled) {
   extern __shared__ __align__(128) uint8_t smem[];  // kStages tiles
   __shared__ __align__(16) float s_ext_all[kGroups][kWarps * 2 * kD];  // see ext_at
@@ -396,19 +419,18 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   if (group == kGroups) {
     // ------------------------------ the fetching warps: descriptors, rotation tables and copies, up to kStages tiles ahead
-    Tile t(first, log_h, m.L);
+    Tile t(jobs, first, n_jobs, per_job, log_h);
     uint32_t rot_job = 0xFFFFFFFFu, stage = 0, phase = 1;  // a fresh barrier passes a wait for the phase before its first
     uint32_t landing = 0, lap = 0;                         // the tile's barrier and the parity of its lap
     int rot_buf = 0;
-    uint32_t left = stalled ? blockIdx.x % (2 * kStages) : 0xFFFFFFFFu;  // tiles until a stalled fetch
-    for (uint32_t item = first; item < last + kGroups; ++item, t.next(H, m.L)) {
+    const uint32_t stop = stalled ? first + blockIdx.x % (2 * kStages) : 0xFFFFFFFFu;  // a stalled fetch ends there
+    for (uint32_t item = first; item < min(last + kGroups, stop); ++item, t.next(jobs, H, m.L, item < last)) {
       const bool end = item >= last;  // an end mark for every group
       const uint8_t* x = nullptr;
       TileDesc td{};
       if (!end) {
         const QuantJob& jb = job_at(jobs, t.job);
         x = static_cast<const uint8_t*>(t.kv ? jb.v : jb.k);
-        if (!x) continue;  // this side of the chunk is not wanted
         const size_t at = (size_t)t.l * layer_elems + (size_t)t.h * (t.kv ? kRows * kD : kD);  // the tile's first element
         const int G = jb.bits == 8 ? 1 : 4;
         x += at * 2;
@@ -417,7 +439,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                             t.kv ? ((size_t)t.l * H + t.h) * kRows * G : ((size_t)t.l * G * H + t.h) * kD, jb.meta16);
         td.kv = t.kv, td.bits = jb.bits, td.meta16 = jb.meta16, td.rot = -1;
       }
-      if (left-- == 0) return;
       if (!mbar_wait(&s_empty[stage], phase, limit)) {
         if (lane == 0) atomicOr(status, DEV_STATUS_WAIT_TIMEOUT);
         asm volatile("cp.async.wait_all;" ::: "memory");  // the copies in flight land before their buffers are given up
@@ -739,21 +760,19 @@ cudaError_t configure_type() {
 }
 
 template <typename Jobs>
-cudaError_t launch_with(const Jobs& jobs, int n_jobs, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl, bool stalled, cudaStream_t st) {
-  const long long n_items = (long long)n_jobs * m.L * 2 * m.Hkv;
-  if (n_items > 0xFFFFFFFFll) return cudaErrorInvalidValue;
+cudaError_t launch_with(const Jobs& jobs, const QuantBatch& b, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl, bool stalled, cudaStream_t st) {
   // one CTA per SM
-  const dim3 grid((unsigned)(n_items < n_sm ? n_items : n_sm)), block(kThreads);
+  const dim3 grid((unsigned)(b.n_tiles < (uint32_t)n_sm ? b.n_tiles : (uint32_t)n_sm)), block(kThreads);
   if (m.dtype == KVB_DT_BF16)
-    return launch_pdl(pdl, quantize_batch_kernel<KVB_DT_BF16, Jobs>, grid, block, kSmemBytes, st, jobs, m, (uint32_t)n_items, inv_freq, status, stalled);
-  return launch_pdl(pdl, quantize_batch_kernel<KVB_DT_F16, Jobs>, grid, block, kSmemBytes, st, jobs, m, (uint32_t)n_items, inv_freq, status, stalled);
+    return launch_pdl(pdl, quantize_batch_kernel<KVB_DT_BF16, Jobs>, grid, block, kSmemBytes, st, jobs, m, b.n_jobs, b.n_tiles, b.per_job, inv_freq, status, stalled);
+  return launch_pdl(pdl, quantize_batch_kernel<KVB_DT_F16, Jobs>, grid, block, kSmemBytes, st, jobs, m, b.n_jobs, b.n_tiles, b.per_job, inv_freq, status, stalled);
 }
 
 template <int N>
-cudaError_t launch_inline(const QuantJob* host_jobs, int n_jobs, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl, bool stalled, cudaStream_t st) {
+cudaError_t launch_inline(const QuantJob* host_jobs, const QuantBatch& b, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl, bool stalled, cudaStream_t st) {
   InlineJobs<N> jobs;
-  memcpy(jobs.d, host_jobs, sizeof(QuantJob) * (size_t)n_jobs);
-  return launch_with(jobs, n_jobs, m, inv_freq, status, n_sm, pdl, stalled, st);
+  memcpy(jobs.d, host_jobs, sizeof(QuantJob) * (size_t)b.n_jobs);
+  return launch_with(jobs, b, m, inv_freq, status, n_sm, pdl, stalled, st);
 }
 
 }  // namespace
@@ -763,16 +782,16 @@ cudaError_t quantize_configure() {
   return e == cudaSuccess ? configure_type<KVB_DT_F16>() : e;
 }
 
-cudaError_t launch_quantize_inline(const QuantJob* host_jobs, int n_jobs, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl, bool stalled,
+cudaError_t launch_quantize_inline(const QuantJob* host_jobs, const QuantBatch& b, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl, bool stalled,
                                    cudaStream_t st) {
-  if (n_jobs <= kSmallInline) return launch_inline<kSmallInline>(host_jobs, n_jobs, m, inv_freq, status, n_sm, pdl, stalled, st);
-  if (n_jobs <= kQuantInline) return launch_inline<kQuantInline>(host_jobs, n_jobs, m, inv_freq, status, n_sm, pdl, stalled, st);
+  if (b.n_jobs <= (uint32_t)kSmallInline) return launch_inline<kSmallInline>(host_jobs, b, m, inv_freq, status, n_sm, pdl, stalled, st);
+  if (b.n_jobs <= (uint32_t)kQuantInline) return launch_inline<kQuantInline>(host_jobs, b, m, inv_freq, status, n_sm, pdl, stalled, st);
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_quantize_table(const QuantJob* table, int n_jobs, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl, bool stalled,
+cudaError_t launch_quantize_table(const QuantJob* table, const QuantBatch& b, const ModelDims& m, const double* inv_freq, uint32_t* status, int n_sm, bool pdl, bool stalled,
                                   cudaStream_t st) {
-  return launch_with(table, n_jobs, m, inv_freq, status, n_sm, pdl, stalled, st);
+  return launch_with(table, b, m, inv_freq, status, n_sm, pdl, stalled, st);
 }
 
 }  // namespace kvb

@@ -409,3 +409,48 @@ def test_long_runs_of_one_side(side, Hkv):
             assert torch.equal(codes, want_codes) and torch.equal(meta, want_meta)
     finally:
         B.kvb_destroy(ctx)
+
+
+@pytest.mark.parametrize("n_jobs,L,Hkv,kv_dtype", [(1000, 1, 1, "bf16"), (250, 3, 2, "fp16"), (40, 12, 4, "fp16"), (3, 36, 16, "bf16")])
+@pytest.mark.parametrize("sides", [("kv", "k", "v", "v", "kv"), ("k",), ("v", "k")])
+def test_jobs_of_every_kind_over_many_tiles(n_jobs, L, Hkv, kv_dtype, sides):
+    """Keys only, values only and both, either code width, compact metadata or not, every job with a position of its own, in
+    one call of many more tiles than a CTA has buffers (and of more rotations than it keeps).  Codes and metadata equal the
+    oracle's bit for bit."""
+    sh = synth.Shape(L=L, Hq=Hkv, Hkv=Hkv, kv_dtype=kv_dtype)
+    dtc = helpers.dt_code(sh)
+    ctx = B.create_for_shape(sh, 0)
+    try:
+        xs = [(_keys(sh, 400 + i), _keys(sh, 500 + i)) for i in range(3)]  # jobs share their inputs, not their outputs
+        dev = [(k.to(DEV), v.to(DEV)) for k, v in xs]
+        oracle_in = [(helpers.bits_of(k), helpers.f64_of(k), helpers.f64_of(v)) for k, v in xs]
+        jobs, spec = [], []
+        for i in range(n_jobs):
+            side, bits, m16, pos = sides[i % len(sides)], 8 if i // 3 % 2 else 4, i % 4 == 1, -1 if i % 7 == 3 else 128 * i
+            mt, G = torch.float16 if m16 else torch.float32, 1 if bits == 8 else 4
+            j = dict(bits=bits, unrotate_from=pos, meta_fp16=m16)
+            for s, x, meta in (("k", dev[i % 3][0], (L, G, Hkv, sh.d, 2)), ("v", dev[i % 3][1], (L, sh.C, Hkv, G, 2))):
+                if s in side:
+                    j.update({s: x, s + "_codes": torch.zeros((L, sh.C, Hkv, sh.d * bits // 8), dtype=torch.uint8, device=DEV), s + "_meta": torch.zeros(meta, dtype=mt, device=DEV)})
+            jobs.append(j)
+            spec.append((side, bits, m16, pos))
+        B.kvb_quantize_chunks(ctx, jobs)
+        B.kvb_last_status(ctx)
+        values = {}  # (input, width, compact) -> the oracle's values
+        for i, (j, (side, bits, m16, pos)) in enumerate(zip(jobs, spec)):
+            kb, k64, v64 = oracle_in[i % 3]
+            gk, gv = (sh.C, sh.d) if bits == 8 else (sh.int4_group, sh.int4_group)
+            if "k" in side and (n_jobs < 100 or i % 9 < 3):
+                got_c, got_m = j["k_codes"].cpu().numpy(), j["k_meta"].float().cpu().numpy()
+                for l in range(L):
+                    u = oracle.unrotate_keys(kb[l], dtc, sh.theta, pos) if pos >= 0 else k64[l]
+                    c, m = oracle.quantize_k(u, bits, gk, meta16=m16)
+                    assert np.array_equal(got_c[l], c) and np.array_equal(got_m[l], m.astype(np.float32)), ("keys", i, l)
+            if "v" in side:
+                key = (i % 3, bits, m16)
+                if key not in values:
+                    r = [oracle.quantize_v(v64[l], bits, gv, meta16=m16) for l in range(L)]
+                    values[key] = np.stack([c for c, _ in r]), np.stack([m for _, m in r]).astype(np.float32)
+                assert np.array_equal(j["v_codes"].cpu().numpy(), values[key][0]) and np.array_equal(j["v_meta"].float().cpu().numpy(), values[key][1]), ("values", i)
+    finally:
+        B.kvb_destroy(ctx)

@@ -11,9 +11,10 @@
 // atomics, so the sum is exact and independent of the order CTAs run in.
 //
 // Bound by HBM reads.  One kernel per combination of sides, so that a side that is not wanted costs
-// neither registers nor arithmetic and its place is taken by a second row, and the next pass's four
-// loads are in flight while a pass is worked on: 4224 positions, keys only, 36 layers of 2 heads
-// (156 MB) 44.9 -> 25.3 us = 6.1 TB/s.
+// neither registers nor arithmetic and its place is taken by a second row.  One side: the next pass's
+// four loads are in flight while a pass is worked on: 4224 positions, keys only, 36 layers of 2 heads
+// (156 MB) 44.9 -> 25.3 us = 6.1 TB/s.  Both sides (40 registers, so the compiler issues a pass's loads
+// where they are used): the same positions, 311 MB, call with selection 70.1 -> 63.6 us.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -29,9 +30,12 @@ namespace kvb {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kTileTokens = 64;
+// Positions of a tile: 64, and for both sides at most 128 (token, head) rows of either.  With 64 positions of 16 heads a CTA
+// is so long that a last wave of a few of them weighs: both sides of 2048 positions, 36 layers, call with selection, 4 / 8 / 16
+// heads 75.8 / 121 / 229 us, in tiles of 128 rows 58.5 / 97.7 / 177; 8192 positions 202 / 375 / 711 and 186 / 344 / 662.
+__host__ __device__ constexpr int tile_tokens(int H, int which) { return which != 3 || H <= 2 ? 64 : 128 / H; }
 
-// grid (tiles over all requests, L).  A tile is kTileTokens consecutive positions of one request.
+// grid (tiles over all requests, L).  A tile is tile_tokens consecutive positions of one request.
 template <int DT, int WHICH, typename Tab>
 __global__ void __launch_bounds__(kThreads)
     deviation_kernel(const __grid_constant__ Tab table, int n_req, ModelDims m, unsigned long long* __restrict__ acc) {
@@ -47,8 +51,8 @@ __global__ void __launch_bounds__(kThreads)
   const ReqDesc rq = reqs[lo];
   const int l = blockIdx.y;
   const int H = m.Hkv;
-  const int t_begin = (tile - rq.tile_offset) * kTileTokens;
-  const int t_end = min(rq.T, t_begin + kTileTokens);
+  const int t_begin = (tile - rq.tile_offset) * tile_tokens(H, WHICH);
+  const int t_end = min(rq.T, t_begin + tile_tokens(H, WHICH));
   const int u_begin = t_begin * H, u_end = t_end * H;  // (token, head) rows of 256 bytes
   const size_t plane = (size_t)rq.T * H * 256;           // bytes of one [T][H][d] plane, d = 128
   const uint8_t* stK = rq.kv_buf + (size_t)(2 * l) * plane;
@@ -65,7 +69,7 @@ __global__ void __launch_bounds__(kThreads)
   const uint8_t* const st = WHICH == 2 ? stK + plane : stK;
   const uint8_t* const fr = WHICH == 2 ? frK + plane : frK;
   const int step = both ? n_hw : 2 * n_hw;
-  // two passes' loads in flight: the next one's are issued before this one's are used
+  // the next pass's loads before this one's are used
   uint4 w[2][4];
   auto load = [&](int u0, uint4 (&x)[4]) {
     const int ua = u0 + s, ub = both ? ua : ua + n_hw;
@@ -99,7 +103,7 @@ __global__ void __launch_bounds__(kThreads)
 
 }  // namespace
 
-int deviation_tile_tokens() { return kTileTokens; }
+int deviation_tile_tokens(int Hkv, int which) { return tile_tokens(Hkv, which); }
 
 cudaError_t launch_deviation(const Table& table, int n_req, int total_tiles, const ModelDims& m, int which,
                              unsigned long long* acc, bool pdl, cudaStream_t st) {

@@ -91,7 +91,7 @@ extern "C" int kvb_deviation_static(int device, const kvb_model_desc* model, con
   store_desc_kernel<<<1, 1, 0, st>>>(d, desc_dev);
   if (cudaGetLastError() != cudaSuccess) return KVB_ERR_CUDA;
   const ModelDims dims{m.L, m.Hq, m.Hkv, m.d, m.chunk_tokens, m.kv_dtype, m.int4_group};
-  const int tiles = (T + deviation_tile_tokens() - 1) / deviation_tile_tokens();
+  const int tile_tokens = deviation_tile_tokens(m.Hkv, which), tiles = (T + tile_tokens - 1) / tile_tokens;
   if (launch_deviation(Table{nullptr, 0, reinterpret_cast<const uint8_t*>(desc_dev)}, 1, tiles, dims, which, acc, false, st) != cudaSuccess) return KVB_ERR_CUDA;
   const int n_terms = m.L * m.Hkv * ((which & 1) + ((which >> 1) & 1));
   finalize_delta_kernel<<<(T + 255) / 256, 256, 0, st>>>(acc, T, (float)(1.0 / (1099511627776.0 * (double)n_terms)), delta);

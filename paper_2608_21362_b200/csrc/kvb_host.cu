@@ -396,7 +396,7 @@ struct SelectExtent {
 // One ReqDesc per request plus the batch's window list (seams, then the sink window, per request).
 int pack_selection(kvb_ctx* c, const kvb_request* reqs, int n_req, const kvb_select_params* p, const kvb_selection* out,
                    ReqDesc* rd, SeamWindow* sw, SelectExtent* ext) {
-  const int tile_tok = deviation_tile_tokens();
+  const int tile_tok = deviation_tile_tokens(c->dims.Hkv, p->which);
   int tiles = 0, tok = 0, n_seams = 0, max_T = 0, max_k = 0;
   for (int r = 0; r < n_req; ++r) {
     const kvb_request& q = reqs[r];

@@ -107,7 +107,7 @@ cudaError_t assemble_configure(size_t max_smem);
 // request descriptors at the start of the table
 cudaError_t launch_deviation(const Table& table, int n_req, int total_tiles, const ModelDims& m, int which,
                              unsigned long long* acc, bool pdl, cudaStream_t st);
-int deviation_tile_tokens();
+int deviation_tile_tokens(int Hkv, int which);  // positions of a tile
 
 // request descriptors at the start of the table, then the window list
 cudaError_t launch_topk(const Table& table, int n_req, const ModelDims& m, int n_terms, int max_T, int max_k, unsigned long long* acc,

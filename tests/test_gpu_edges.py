@@ -472,3 +472,9 @@ def test_tables_of_every_size_reach_the_selection_and_the_importance(n_req):
                 assert torch.equal(a, b)
     finally:
         B.kvb_destroy(ctx)
+
+
+@pytest.mark.parametrize("Hkv,T", [(4, 31), (4, 32), (4, 33), (8, 15), (8, 16), (8, 17), (16, 7), (16, 8), (16, 9), (16, 137)])
+def test_deviation_of_both_sides_on_short_tiles(Hkv, T):
+    """Keys and values of four heads and more go in tiles of 128 rows: full, one position short and one over."""
+    test_deviation_kernel_sides_and_ragged_tiles("bf16", Hkv, 3, T)

@@ -6,15 +6,16 @@
 // One launch quantises a batch of chunks.  Work unit: a tile of 128 rows x 128 channels (32 KB):
 //   keys    the 128 tokens of one (chunk, layer, KV head)
 //   values  128 consecutive (token, head) rows of one (chunk, layer)
-// One persistent CTA per SM walks a contiguous range of tiles: three groups of eight warps work on a tile each,
+// One persistent CTA per SM walks a contiguous range of the wanted tiles: three groups of eight warps work on a tile each,
 // four more warps fetch ahead into a ring of five tile buffers (one bulk copy where the tile is contiguous, cp.async by
 // token rows for one head of several: a bulk copy per 256-byte row took twice the time), and hand over through mbarriers,
 // so that loads go on while tiles are in work.  Bound by the instructions of the code decision and, for plain values, by
-// HBM.  64 chunks, one side only, against one CTA of eight warps per 64 KB tile loading and computing in turn: int8 values
-// 41 us (36 us at the copy rate), int4 values 42, int8 keys 50, int4 keys 51, rotated int4 keys 64; both sides of a
-// 16K-token prompt to int4, position-free: 221 -> 202 us, of a 2K-token prompt to int8: 29.4 -> 24.5 us (one launch
-// instead of two: up to 256 jobs travel as the kernel's argument).  Two groups, with registers to spare, measured 3-8 %
-// slower; consumer warps fetching for themselves likewise.
+// HBM.  64 chunks of 36 layers and 2 heads, one side only, before (one CTA of eight warps per 64 KB tile, loading and
+// computing in turn) and now: int8 values 53.0 / 39.1 us (36 us at the copy rate), int4 values 61.5 / 40.7, int8 keys
+// 52.7 / 44.5, int4 keys 54.7 / 46.4, rotated int4 keys 70.8 / 61.2; both sides of a 16K-token prompt to int4,
+// position-free and compact: 216 / 182, of a 2K-token prompt to int8: 29.6 / 23.1 (one launch instead of two: up to 256
+// jobs travel as the kernel's argument).  Two groups, with registers to spare, measured 3-8 % slower; consumer warps
+// fetching for themselves likewise.
 //   keys    a thread owns a quad of neighbouring channels, their rotation partners 64 channels on, and eight tokens.
 //           Without the rotation the extremes are taken on the 16-bit values, two per instruction.  With `unrotate`
 //           every key is first rotated back by R_theta^(-orig_pos) (Rotary Positional Embeddings, Eq. 3), so that the

@@ -10,7 +10,6 @@
 namespace kvb {
 
 struct TableAddress {
-  static constexpr bool kInline = false;
   const uint8_t* p;
 #ifdef __CUDACC__
   __device__ __forceinline__ const uint8_t* base() const { return p; }
@@ -18,7 +17,6 @@ struct TableAddress {
 };
 template <size_t BYTES>
 struct alignas(64) TableBytes {
-  static constexpr bool kInline = true;
   uint8_t b[BYTES];
 #ifdef __CUDACC__
   __device__ __forceinline__ const uint8_t* base() const { return b; }

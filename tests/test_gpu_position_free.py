@@ -128,8 +128,8 @@ def test_batched_quantiser_codes_bit_exact(kv_dtype, Hkv):
                 k[:, :, :, 9] = 1.0
                 k[:, 64:, :, 9] = 1.0 + 2.0 ** -7
                 v[:, 7, :, ::2] = 3.0e4 if kv_dtype == "fp16" else 1.0e30
-            if i >= 8:  # integers in [0, 2 * levels] with both ends in every group: scale 2, the odd ones tie, far
-                # more of them than the kernel's list of places to redo with the IEEE division holds
+            if i >= 8:  # integers in [0, 2 * levels] with both ends in every group: scale 2, the odd ones tie, and the
+                # quotient without a division has to round them as the division would
                 top = 2 * ((1 << bits) - 1)
                 g = torch.Generator().manual_seed(300 + i)
                 k = torch.randint(0, top // 2 + 1, (sh.L, sh.C, Hkv, sh.d), generator=g).float()

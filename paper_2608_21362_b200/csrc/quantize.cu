@@ -84,8 +84,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32
   }
   return false;
 }
-// a group's own barrier
-__device__ __forceinline__ void group_sync(int group) { asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(kWarps * 32) : "memory"); }
 // The same for a single lane, whose answer may differ from its neighbours': without the vote 58 chunks of keys and values to
 // int4 take 73.2 instead of 73.9 us.
 __device__ __forceinline__ bool mbar_wait_lane(uint64_t* bar, uint32_t parity, uint32_t limit) {
@@ -95,6 +93,8 @@ __device__ __forceinline__ bool mbar_wait_lane(uint64_t* bar, uint32_t parity, u
   }
   return false;
 }
+// a group's own barrier
+__device__ __forceinline__ void group_sync(int group) { asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(kWarps * 32) : "memory"); }
 // After a lane's wait for its group's tile has run out: true if the tile has landed after all, false if the wait has run out
 // for every lane of the group (`gave_up` counts them; all of them is final).  So the lanes of a group leave together or go on
 // together, and none is left waiting for another in group_sync or a shuffle.  It ends: a tile that one lane has seen stays

@@ -218,8 +218,10 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
   const bool dev_on = DEV && acc != nullptr && (which & (kv ? 2 : 1));
   const bool norm_on = NORM && kv == 0;
   // The warps read the fresh rows a token pair at a time, one pair ahead (registers allow no more), which keeps too few bytes
-  // in flight for HBM: one request brings this CTA's whole block of them into L2 first.  (See launch_assemble for when.)
-  if (DEV && dev_on && fresh_ahead && cd.mode != KVB_MODE_FRESH && tid == 0) l2_prefetch(cd.fresh + dst_off * 2, (uint32_t)out_bytes);
+  // in flight for HBM.  So every half-warp also has the pair after that on its way into L2 (prefetch_fresh); with the norms,
+  // where the loop has no registers left for it, one request brings this CTA's whole block first (see launch_assemble for when).
+  constexpr bool kPairsAhead = DEV && !NORM;
+  if (NORM && dev_on && fresh_ahead && cd.mode != KVB_MODE_FRESH && tid == 0) l2_prefetch(cd.fresh + dst_off * 2, (uint32_t)out_bytes);
   unsigned long long* acc_tok = dev_on ? acc + cd.tok_offset + cd.new_pos + tb : nullptr;  // this CTA's first token
   auto norm_out = [&]() { return norm_sums + ((size_t)ci * m.L + l) * split + part_id; };  // this CTA's slot
   float norm_part = 0.f;  // lanes 0 and 8 of each half-warp: norms of the rows they reduced
@@ -374,13 +376,22 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
         if ((ln & 7) == 0 && (!heads_paired || s == 0)) atomicAdd(acc_tok + t + (ln >> 3), (unsigned long long)fx);
       }
     };
+    // starts the fresh rows of tokens t and t + 1 on their way into L2: four 128-byte lines, a lane of the half-warp each
+    auto prefetch_fresh = [&](int t) {
+      if (ln < 4) {
+        const uint8_t* p = fresh_rows + ((size_t)(((t + (ln >> 1)) << log_h) + h) << 8) + 128 * (ln & 1);
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(p) : "memory");
+      }
+    };
     // the row loop shared by keys and values: two tokens per pass, the next pair's fresh words in flight
     auto run_rows = [&](auto&& one_row) {
       uint2 fr[4] = {}, fr_next[4] = {};
       if (dev_on) load_fresh(t0, fr);
+      if (kPairsAhead && dev_on && tok_per > 2) prefetch_fresh(t0 + 2);
       for (int tt = 0; tt < tok_per; tt += 2) {  // tok_per is even and a pair never straddles a part
         const int t = t0 + tt;
         if (!part_ready(t)) break;
+        if (kPairsAhead && dev_on && tt + 4 < tok_per) prefetch_fresh(t + 4);
         if (dev_on && tt + 2 < tok_per) load_fresh(t + 2, fr_next);
         uint2 wl0, wh0, wl1, wh1;
         one_row(t, wl0, wh0);
@@ -615,10 +626,12 @@ cudaError_t launch_assemble(const ChunkDesc* chunks, int n_chunks, const float2*
                             size_t smem_bytes, uint32_t* status, int which, unsigned long long* acc, double* norm_sums,
                             int n_sm, bool pdl, cudaStream_t st) {
   const unsigned grid = (unsigned)n_chunks * m.L * 2 * assemble_split(m.Hkv);
-  // From four waves of CTAs on the fresh rows are fetched into L2 in whole blocks.  One prompt, 36 layers, 2 KV heads, stitch
-  // and selection, without / with: 8192 tokens int4 166 / 152 us, 6144 int8 128 / 122, mixed 129 / 125, 4096 int8 93.0 / 91.1;
-  // 24 short prompts 482 / 442; 3200 tokens of 4 heads 134 / 125.  Below, all CTAs start together and their requests only
-  // stand in the way of the codes: 2048 mixed 56.3 / 58.4, 1024 int8 36.8 / 37.9.
+  // Fresh rows.  Without the norms a pair of tokens goes into L2 ahead of the pair that is being loaded: one prompt, 36
+  // layers, 2 KV heads, stitch and selection, with nothing ahead / so: 1024 tokens mixed 33.2 / 31.1 us, 2048 int8 51.0 /
+  // 47.4, mixed 52.2 / 49.4, int4 50.7 / 48.1; with whole blocks requested at once / so: 3200 tokens of 4 heads 121.5 /
+  // 116.6, 8192 int4 146.8 / 146.5.  (Four or five pairs ahead: 2048 int8 48.9.)  With the norms that costs registers (24
+  // short prompts 444 -> 456), and from four waves of CTAs on whole blocks are requested (482 -> 442); below, all CTAs start
+  // together and such requests only stand in the way of the codes.
   const bool fresh_ahead = grid >= 4u * kCtasPerSm * (unsigned)n_sm;
   const bool dev = acc != nullptr && (which & 3);
   if (!dev) which = 0, acc = nullptr;

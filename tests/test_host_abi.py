@@ -247,3 +247,21 @@ def test_validator_agrees_with_the_stated_rules_on_random_tables():
         assert got == _expected_status(T, chunks, kv_ptr, fresh_ptr, need_payload), (buf.value, T, chunks)
 
     run()
+
+
+def test_library_is_rebuilt_after_a_change_in_any_source(tmp_path, monkeypatch):
+    """Every file that goes into the library makes it stale, the headers that only kernels include too."""
+    from paper_2608_21362_b200 import build
+
+    files = [os.path.join(d, n) for d in (build.CSRC, os.path.join(build.ROOT, "include")) for n in sorted(os.listdir(d))]
+    assert {os.path.splitext(f)[1] for f in files} == {".cu", ".cuh", ".h"}
+    so = tmp_path / "libkvb.so"
+    so.write_bytes(b"")
+    newest = max(os.path.getmtime(f) for f in files)
+    os.utime(so, (newest + 10, newest + 10))
+    monkeypatch.setattr(build, "LIB", str(so))
+    assert not build._stale()
+    getmtime = os.path.getmtime
+    for changed in files:
+        monkeypatch.setattr(os.path, "getmtime", lambda p: newest + 20 if os.path.samefile(p, changed) else getmtime(p))
+        assert build._stale(), changed

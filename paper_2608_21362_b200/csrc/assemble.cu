@@ -190,7 +190,7 @@ template <typename OutT, bool DEV, bool NORM>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
     assemble_kernel(const ChunkDesc* __restrict__ chunks, const float2* __restrict__ cs_table, ModelDims m,
                     uint32_t* __restrict__ status, int which, unsigned long long* __restrict__ acc,
-                    double* __restrict__ norm_sums, bool fresh_ahead) {
+                    double* __restrict__ norm_sums, bool block_ahead) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ __align__(8) uint64_t bars[kParts + 1];
   __shared__ float s_norm[kThreads / 32];
@@ -217,11 +217,12 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 
   const bool dev_on = DEV && acc != nullptr && (which & (kv ? 2 : 1));
   const bool norm_on = NORM && kv == 0;
-  // The warps read the fresh rows a token pair at a time, one pair ahead (registers allow no more), which keeps too few bytes
-  // in flight for HBM.  So every half-warp also has the pair after that on its way into L2 (prefetch_fresh); with the norms,
-  // where the loop has no registers left for it, one request brings this CTA's whole block first (see launch_assemble for when).
+  // The staged row loop reads the fresh rows a token pair at a time, one pair ahead (registers allow no more), which keeps too
+  // few bytes in flight for HBM.  Without the norms every half-warp there also has the pair after that on its way into L2
+  // (prefetch_fresh); with the norms the loop has no registers left for it, and one request brings this CTA's whole block
+  // first.  Rows that are copied have enough loads of their own in flight.  (launch_assemble has the figures.)
   constexpr bool kPairsAhead = DEV && !NORM;
-  if (NORM && dev_on && fresh_ahead && cd.mode != KVB_MODE_FRESH && tid == 0) l2_prefetch(cd.fresh + dst_off * 2, (uint32_t)out_bytes);
+  if (NORM && dev_on && block_ahead && cd.mode != KVB_MODE_FRESH && tid == 0) l2_prefetch(cd.fresh + dst_off * 2, (uint32_t)out_bytes);
   unsigned long long* acc_tok = dev_on ? acc + cd.tok_offset + cd.new_pos + tb : nullptr;  // this CTA's first token
   auto norm_out = [&]() { return norm_sums + ((size_t)ci * m.L + l) * split + part_id; };  // this CTA's slot
   float norm_part = 0.f;  // lanes 0 and 8 of each half-warp: norms of the rows they reduced
@@ -376,7 +377,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
         if ((ln & 7) == 0 && (!heads_paired || s == 0)) atomicAdd(acc_tok + t + (ln >> 3), (unsigned long long)fx);
       }
     };
-    // starts the fresh rows of tokens t and t + 1 on their way into L2: four 128-byte lines, a lane of the half-warp each
+    // Starts the fresh rows of tokens t and t + 1 on their way into L2: their four 128-byte pieces, a lane of the half-warp
+    // each.  A piece is one line when `fresh` lies on a 128-byte boundary; otherwise (16 bytes are what is asked for) its end
+    // is in the next piece's line, and the last one of a run comes with the load itself.
     auto prefetch_fresh = [&](int t) {
       if (ln < 4) {
         const uint8_t* p = fresh_rows + ((size_t)(((t + (ln >> 1)) << log_h) + h) << 8) + 128 * (ln & 1);
@@ -387,7 +390,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
     auto run_rows = [&](auto&& one_row) {
       uint2 fr[4] = {}, fr_next[4] = {};
       if (dev_on) load_fresh(t0, fr);
-      if (kPairsAhead && dev_on && tok_per > 2) prefetch_fresh(t0 + 2);
+      if (kPairsAhead && dev_on) prefetch_fresh(t0 + 2);  // tok_per is 8 (one head) or 16
       for (int tt = 0; tt < tok_per; tt += 2) {  // tok_per is even and a pair never straddles a part
         const int t = t0 + tt;
         if (!part_ready(t)) break;
@@ -626,24 +629,32 @@ cudaError_t launch_assemble(const ChunkDesc* chunks, int n_chunks, const float2*
                             size_t smem_bytes, uint32_t* status, int which, unsigned long long* acc, double* norm_sums,
                             int n_sm, bool pdl, cudaStream_t st) {
   const unsigned grid = (unsigned)n_chunks * m.L * 2 * assemble_split(m.Hkv);
-  // Fresh rows.  Without the norms a pair of tokens goes into L2 ahead of the pair that is being loaded: one prompt, 36
-  // layers, 2 KV heads, stitch and selection, with nothing ahead / so: 1024 tokens mixed 33.2 / 31.1 us, 2048 int8 51.0 /
-  // 47.4, mixed 52.2 / 49.4, int4 50.7 / 48.1; with whole blocks requested at once / so: 3200 tokens of 4 heads 121.5 /
-  // 116.6, 8192 int4 146.8 / 146.5.  (Four or five pairs ahead: 2048 int8 48.9.)  With the norms that costs registers (24
-  // short prompts 444 -> 456), and from four waves of CTAs on whole blocks are requested (482 -> 442); below, all CTAs start
-  // together and such requests only stand in the way of the codes.
-  const bool fresh_ahead = grid >= 4u * kCtasPerSm * (unsigned)n_sm;
+  // Fresh rows, the times of stitch and selection alone (calls back to back over inputs larger than L2, both forms in turn,
+  // medians of 13 blocks that differ by 0.3 %, 1.5 % for the batches; 36 layers, 2 KV heads, three quarters cached): whole
+  // blocks requested from four waves of CTAs on and nothing below / the pair ahead in the staged loop:
+  //   1024 mixed 32.4 / 30.5 us, 2048 int8 50.9 / 47.2, mixed 51.6 / 49.4, int4 50.5 / 47.7, 4096 int8 87.6 / 80.4, mixed
+  //   89.6 / 83.7, 6144 mixed 121.5 / 115.6, 8192 mixed 152.5 / 147.4, int4 146.5 / 146.6, 16384 mixed 284.8 / 274.5, 3200 of
+  //   4 heads 121.8 / 116.6, 8 ragged prompts 825 / 796; the other way only large int4 prompts, whose loop is short of issue
+  //   slots: 8832 of one head, keys alone 74.0 / 74.8, 8192 with `fresh` off the 128-byte boundaries 155.9 / 157.0.
+  // (Four or five pairs ahead: 2048 int8 48.9.)  In a whole step the attention's clock under the power cap gives most of it
+  // back: 2048 int8 with the attention 249.3 / 248.7, 3200 of 4 heads 603.6 / 602.1, not beyond the spread.
+  // Copied rows get no request: their loop has four 16-byte loads per thread in flight, and with their blocks requested as
+  // well 4096 mixed goes from 83.7 to 84.8, 4096 of 16-bit chunks from 85.8 to 87.5, 8192 of them, values alone, from 135.2
+  // to 136.3 (135.9 with whole blocks for all).  With the norms the pair ahead costs registers (24 short prompts 444 -> 456),
+  // and whole blocks are requested (482 -> 442) from four waves on; below, all CTAs start together and such requests only
+  // stand in the way of the codes.
+  const bool block_ahead = norm_sums && grid >= 4u * kCtasPerSm * (unsigned)n_sm;
   const bool dev = acc != nullptr && (which & 3);
   if (!dev) which = 0, acc = nullptr;
   const dim3 g(grid), b(kThreads);
   if (m.dtype == KVB_DT_BF16) {
-    if (norm_sums) return launch_pdl(pdl, assemble_kernel<__nv_bfloat16, true, true>, g, b, smem_bytes, st, chunks, cs_table, m, status, which, acc, norm_sums, fresh_ahead);
-    if (dev) return launch_pdl(pdl, assemble_kernel<__nv_bfloat16, true, false>, g, b, smem_bytes, st, chunks, cs_table, m, status, which, acc, norm_sums, fresh_ahead);
-    return launch_pdl(pdl, assemble_kernel<__nv_bfloat16, false, false>, g, b, smem_bytes, st, chunks, cs_table, m, status, which, acc, norm_sums, fresh_ahead);
+    if (norm_sums) return launch_pdl(pdl, assemble_kernel<__nv_bfloat16, true, true>, g, b, smem_bytes, st, chunks, cs_table, m, status, which, acc, norm_sums, block_ahead);
+    if (dev) return launch_pdl(pdl, assemble_kernel<__nv_bfloat16, true, false>, g, b, smem_bytes, st, chunks, cs_table, m, status, which, acc, norm_sums, block_ahead);
+    return launch_pdl(pdl, assemble_kernel<__nv_bfloat16, false, false>, g, b, smem_bytes, st, chunks, cs_table, m, status, which, acc, norm_sums, block_ahead);
   }
-  if (norm_sums) return launch_pdl(pdl, assemble_kernel<__half, true, true>, g, b, smem_bytes, st, chunks, cs_table, m, status, which, acc, norm_sums, fresh_ahead);
-  if (dev) return launch_pdl(pdl, assemble_kernel<__half, true, false>, g, b, smem_bytes, st, chunks, cs_table, m, status, which, acc, norm_sums, fresh_ahead);
-  return launch_pdl(pdl, assemble_kernel<__half, false, false>, g, b, smem_bytes, st, chunks, cs_table, m, status, which, acc, norm_sums, fresh_ahead);
+  if (norm_sums) return launch_pdl(pdl, assemble_kernel<__half, true, true>, g, b, smem_bytes, st, chunks, cs_table, m, status, which, acc, norm_sums, block_ahead);
+  if (dev) return launch_pdl(pdl, assemble_kernel<__half, true, false>, g, b, smem_bytes, st, chunks, cs_table, m, status, which, acc, norm_sums, block_ahead);
+  return launch_pdl(pdl, assemble_kernel<__half, false, false>, g, b, smem_bytes, st, chunks, cs_table, m, status, which, acc, norm_sums, block_ahead);
 }
 
 }  // namespace kvb

@@ -174,3 +174,39 @@ def test_random_ragged_batches_through_the_one_pass_path_and_attention(seed):
             assert not outs[i][:, n:].any()
     finally:
         B.kvb_destroy(ctx)
+
+
+@pytest.mark.parametrize("importance", [False, True])
+@pytest.mark.parametrize("Hkv,L", [(1, 3), (16, 12)])  # the shortest run of tokens per half-warp; a grid of more than four waves
+def test_fused_on_tensors_at_sixteen_byte_offsets(Hkv, L, importance):
+    """The fresh rows are asked for ahead in 128-byte pieces, the header asks for 16-byte alignment: the
+    same bits from tensors at odd multiples of 16 bytes, the two-call path's deviation and the
+    stand-alone scores (float32 sums in another order: 1e-6 and 2e-6 as elsewhere)."""
+    wl = _mixed_workload(Hkv, Hkv, "bf16", L=L)
+    reqs = prepare(wl)
+    (r,) = reqs
+    n_ch = len(r.chunks)
+    ctx = B.create_for_shape(wl.shape, 0)
+    try:
+        run_assemble(ctx, reqs)
+        plain = r.kv_buf.view(torch.int16).clone()
+        got = []
+        for offset in (0, 8, 24):  # elements of two bytes
+            for name in ("fresh", "kv_buf"):
+                t = getattr(r, name)
+                pool = torch.zeros(t.numel() + 64, dtype=t.dtype, device=DEV)
+                assert pool.data_ptr() % 128 == 0
+                setattr(r, name, pool[offset : offset + t.numel()].view(t.shape).copy_(t))
+            r.importance = torch.zeros(n_ch, device=DEV) if importance else None
+            tbl, sel, _ = run_fused(ctx, wl, reqs)
+            assert torch.equal(r.kv_buf.view(torch.int16), plain)
+            got.append((sel.delta[0], sel.rank[0], sel.sel[0], sel.n_sel, *([r.importance] if importance else [])))
+        assert all(torch.equal(a, b) for other in got[1:] for a, b in zip(got[0], other))
+        two, _, _ = run_select(ctx, wl, reqs, tbl, use_oracle_buffer=False)
+        assert float((two.delta[0] - got[0][0]).abs().max()) <= 1e-6
+        if importance:
+            alone = torch.zeros(n_ch, device=DEV)
+            B.kvb_chunk_importance(ctx, tbl, [alone])
+            assert float(((alone - r.importance) / alone).abs().max()) <= 2e-6
+    finally:
+        B.kvb_destroy(ctx)
